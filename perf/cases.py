@@ -24,7 +24,8 @@ import torch
 import paper_2303_07293_gb300 as st
 
 FWHM = 3.0
-CAPACITY = 1 << 17   # detections (tracks) that a program keeps room for
+CAPACITY = 1 << 20   # detections that a program keeps room for
+MAX_TRACKS = 1 << 17
 
 
 def _search(name, w, h, n, nv, hours, step_px, **kw):
@@ -245,7 +246,7 @@ def prepare(case, seed):
     out = out[:n]
     if kind == "tracks":
         s["cands"] = out
-        s["tracks"] = np.zeros(CAPACITY, st.TRACK_DTYPE)
+        s["tracks"] = np.zeros(MAX_TRACKS, st.TRACK_DTYPE)
     else:
         snr = out[:, 5].view(torch.float32)
         top = torch.sort(snr, descending=True, stable=True).indices
@@ -297,7 +298,7 @@ def run(state):
         return dict(J=J.detach(), grad=theta.grad)
     if kind == "tracks":
         rec = state["plan"].link_tracks(state["cands"])
-        state["tracks"][:len(rec)] = rec[:CAPACITY]
+        state["tracks"][:len(rec)] = rec[:MAX_TRACKS]
         return dict(_cols(state["tracks"]), n=len(rec))
     if kind == "median":
         out, med = st.median_subtract(state["frames"], with_median=True)
