@@ -502,11 +502,50 @@ __device__ __forceinline__ float normalize_pair(float r, const NormFrame& f, boo
   return none ? 0.0f : v;
 }
 
+// The warps' largest value into *absmax (values >= 0 order as their bits).
+__device__ __forceinline__ void put_max(float top, unsigned* absmax) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+  if ((threadIdx.x & 31) == 0 && m > *absmax) atomicMax(absmax, m);
+}
+
+__global__ void __launch_bounds__(256)
+    k_absmax(const float* __restrict__ x, int64_t n, unsigned* __restrict__ absmax) {
+  const int64_t head = min(n, (int64_t)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15) / 4);
+  const float4* v = reinterpret_cast<const float4*>(x + head);
+  const int64_t nv = (n - head) / 4, tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  float top = 0.0f;
+  if (tid < head) top = fabsf(x[tid]);
+  if (tid < n - head - 4 * nv) top = fmaxf(top, fabsf(x[head + 4 * nv + tid]));
+#pragma unroll 4
+  for (int64_t j = tid; j < nv; j += (int64_t)gridDim.x * blockDim.x) {
+    const float4 q = __ldg(v + j);
+    top = fmaxf(top, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+  }
+  put_max(top > 0.0f ? top : 0.0f, absmax);  // (a NaN head or tail counts as 0)
+}
+
+__global__ void k_run_margins(const FieldDev* __restrict__ fds, int n,
+                              const unsigned* __restrict__ absmax, float* __restrict__ margin,
+                              int* __restrict__ use) {
+  const int f = threadIdx.x;
+  bool ok = true;
+  if (f < n) {
+    const FieldDev& d = fds[f];
+    // (a 16-bit value may be larger than the value it was rounded from)
+    const float m = run_margin(1.01f * __uint_as_float(absmax[f]), d.N, d.thr[d.N]);
+    margin[f] = m;
+    ok = run_margin_ok(m, d.nmin, d.thr[d.nmin]);
+  }
+  const int all = __syncthreads_and(ok);
+  if (f == 0) *use = all;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_normalize_store(const float* __restrict__ raw, int64_t npix, int normalize, float cr_clip,
                       const SkyState* __restrict__ state, T* __restrict__ cube,
-                      double* __restrict__ mu_out, double* __restrict__ sigma_out) {
+                      double* __restrict__ mu_out, double* __restrict__ sigma_out,
+                      unsigned* __restrict__ absmax) {
   const int i = blockIdx.y;
   const float* x = raw + (int64_t)i * npix;
   T* o = cube + (int64_t)i * npix;
@@ -532,6 +571,7 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   const NormFrame f = s_f;
   auto clipped = [&](float v) { return cr_clip > 0.0f && fabsf(v) > cr_clip ? 0.0f : v; };
+  float top = 0.0f;
   // four pixels; the FP64 formula sits behind one branch
   auto values = [&](float4 r) {
     if (!normalize) return r;
@@ -558,6 +598,8 @@ __global__ void __launch_bounds__(256)
     for (int64_t j = first; j < npix / 4; j += stride) {
       const float4 r = __ldcs(reinterpret_cast<const float4*>(x) + j);
       const float4 w = values(r);
+      if (absmax)
+        top = fmaxf(top, fmaxf(fmaxf(fabsf(w.x), fabsf(w.y)), fmaxf(fabsf(w.z), fabsf(w.w))));
       alignas(16) T v[4] = {to_store<T>(w.x), to_store<T>(w.y), to_store<T>(w.z),
                             to_store<T>(w.w)};
       if constexpr (sizeof(T) == 4)
@@ -565,6 +607,7 @@ __global__ void __launch_bounds__(256)
       else
         reinterpret_cast<uint2*>(o)[j] = *reinterpret_cast<const uint2*>(v);
     }
+    if (absmax) put_max(top, absmax);
     return;
   }
   for (int64_t j = first; j < npix; j += 4 * stride) {
@@ -574,11 +617,14 @@ __global__ void __launch_bounds__(256)
     r.z = j + 2 * stride < npix ? x[j + 2 * stride] : 0.0f;
     r.w = j + 3 * stride < npix ? x[j + 3 * stride] : 0.0f;
     r = values(r);
+    if (absmax)
+      top = fmaxf(top, fmaxf(fmaxf(fabsf(r.x), fabsf(r.y)), fmaxf(fabsf(r.z), fabsf(r.w))));
     o[j] = to_store<T>(r.x);
     if (j + stride < npix) o[j + stride] = to_store<T>(r.y);
     if (j + 2 * stride < npix) o[j + 2 * stride] = to_store<T>(r.z);
     if (j + 3 * stride < npix) o[j + 3 * stride] = to_store<T>(r.w);
   }
+  if (absmax) put_max(top, absmax);
 }
 
 }  // namespace
@@ -600,7 +646,7 @@ size_t sky_partial_doubles(int N) {
 
 int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float cr_clip,
                      int storage, void* cube, double* mu, double* sigma, double* partial,
-                     cudaStream_t s) {
+                     unsigned* absmax, cudaStream_t s) {
   int launches = 0;
   SkyPartial* parts = reinterpret_cast<SkyPartial*>(partial);
   SkyState* state = reinterpret_cast<SkyState*>(parts + (size_t)N * kSkyBlocks);
@@ -621,18 +667,31 @@ int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float
   switch (storage) {
     case ST_F32:
       k_normalize_store<float><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                 (float*)cube, mu, sigma);
+                                                 (float*)cube, mu, sigma, absmax);
       break;
     case ST_F16:
       k_normalize_store<__half><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                  (__half*)cube, mu, sigma);
+                                                  (__half*)cube, mu, sigma, absmax);
       break;
     default:
       k_normalize_store<__nv_bfloat16><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                         (__nv_bfloat16*)cube, mu, sigma);
+                                                         (__nv_bfloat16*)cube, mu, sigma,
+                                                         absmax);
       break;
   }
   return launches + 1;
+}
+
+int launch_absmax(const float* x, int64_t n, unsigned* absmax, cudaStream_t s) {
+  const int64_t blocks = std::min((int64_t)8 * 152, (n + 4095) / 4096);
+  k_absmax<<<(unsigned)std::max((int64_t)1, blocks), 256, 0, s>>>(x, n, absmax);
+  return 1;
+}
+
+int launch_run_margins(const FieldDev* fds, int n, const unsigned* absmax, float* margin, int* use,
+                       cudaStream_t s) {
+  k_run_margins<<<1, 256, 0, s>>>(fds, n, absmax, margin, use);
+  return 1;
 }
 
 }  // namespace st

@@ -58,6 +58,7 @@
 #include "st_internal.h"
 #include "st_pending.cuh"
 #include "st_sample.cuh"
+#include "st_stack_field.cuh"
 #include "st_tma.cuh"
 
 namespace st {
@@ -65,64 +66,27 @@ namespace st {
 namespace {
 
 constexpr int kXV = 8;           // x-velocities per block, one per warp (within a row group)
-constexpr int kMB = 4;           // y-velocities per block (staircase group)
-constexpr int kTX = 32;          // pixel tile width; its height is the variant's KY
 // Storage traits: TMA box width (elements; 16-byte rows) and the largest
 // column offset of a warp (16-bit storage: the 4-bit packing's limit).
 template <typename T>
 struct Store;
 template <>
-struct Store<float> {
+struct Store<float> : StoreType<float> {
   static constexpr int kBoxW = 40;
-  static constexpr CUtensorMapDataType kTma = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  __device__ static float f(float v) { return v; }
 };
 template <>
-struct Store<__half> {
+struct Store<__half> : StoreType<__half> {
   static constexpr int kBoxW = 48, kOColMax = 15;
-  static constexpr CUtensorMapDataType kTma = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  __device__ static float f(__half v) { return __half2float(v); }
 };
 template <>
-struct Store<__nv_bfloat16> {
+struct Store<__nv_bfloat16> : StoreType<__nv_bfloat16> {
   static constexpr int kBoxW = 48, kOColMax = 15;
-  static constexpr CUtensorMapDataType kTma = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-  __device__ static float f(__nv_bfloat16 v) { return __bfloat162float(v); }
 };
-constexpr int kSuper = 4;        // pixel tiles per super-tile side (L2 locality)
-constexpr uint64_t kWaitNs = 2000000000ull;  // wait limit: 2 s of wall-clock time
-constexpr unsigned kProducerSleepNs = 128;  // producer back-off between polls
-constexpr int kPatterns = 15;
+constexpr uint64_t kWaitNs = kStackWaitNs;
 constexpr int kX2Wide = 8;       // extra box columns for 16 x-velocities a half
 // table maxima: column offset in a tile, pattern id, shift spread, column
 // offset in a pair of tiles
 constexpr int kMaxes = 4;
-
-// One field of a launch: geometry, per-frame tile tables and thresholds.
-struct FastField {
-  int W, H, N, nvx, nvy, nA, nB, nmin, field;
-  const int4* xt;   // [N][nA]: box x offset, packed 4-bit column offsets, min shift, max shift
-  const int4* yt;   // [N][nB]: min shift, max shift, pattern id, 0
-  const unsigned char* pat;  // [N][nB] staircase pattern ids
-  const int32_t* sx;
-  const int32_t* sy;
-  const float* fx;   // bilinear: FP32 fractions [N][nvx], [N][nvy]
-  const float* fy;
-  const float4* fxt;  // bilinear: [N][nA][2] x-fractions of a velocity tile's 8 x-velocities
-  const float4* fyt;  // bilinear: [N][nB] y-fractions of its 4 y-velocities
-  const float* thr;
-  // coverage prefix tables: for velocity a, covx[a * cov_len + s - cov_xmin[a]]
-  // = number of frames with sx(i, a) <= s (likewise y)
-  const int* covx;
-  const int* covy;
-  const int* cov_xmin;
-  const int* cov_xmax;
-  const int* cov_ymin;
-  const int* cov_ymax;
-  int cov_len;
-};
-
-constexpr int kMaxFields = 256;
 
 struct FastArgs {
   const FastField* ff[kMaxFields];    // the launch's fields, longest first (device)
@@ -135,20 +99,8 @@ struct FastArgs {
   Counters* ctr;
   float* dump_S;    // optional [nvx*nvy][H][W] of a single field (tests)
   int32_t* dump_C;
+  const int* d_skip;  // non-zero: the run kernel has done the work (or NULL)
 };
-
-// Pattern id -> row offsets of the 4 y-velocities (min offset 0).
-// ids 0..7: non-decreasing, steps (id&1, id>>1&1, id>>2&1);
-// ids 8..14: non-increasing, steps of t = id - 7 read from the other end.
-__host__ __device__ constexpr int pat_off(int id, int j) {
-  if (id < 8) {
-    int s1 = id & 1, s2 = (id >> 1) & 1, s3 = (id >> 2) & 1;
-    return j == 0 ? 0 : j == 1 ? s1 : j == 2 ? s1 + s2 : s1 + s2 + s3;
-  }
-  int t = id - 7;
-  int t1 = t & 1, t2 = (t >> 1) & 1, t3 = (t >> 2) & 1;
-  return j == 0 ? t1 + t2 + t3 : j == 1 ? t2 + t3 : j == 2 ? t3 : 0;
-}
 
 __device__ int pattern_of(const int (&c)[kMB]) {
   for (int id = 0; id < kPatterns; ++id) {
@@ -315,13 +267,6 @@ __device__ __forceinline__ void add_pattern_bl(float2 (&acc)[kMB][KY / 2], const
   add_bl_column<KY, pat_off(ID, 3)>(acc[3], gy[3], fy[3], hp);
 }
 
-// Number of frames whose shift s satisfies lo <= s <= hi, from a prefix table.
-__device__ __forceinline__ int count_shifts(const int* pre, int smin, int smax, int N, int lo,
-                                            int hi) {
-  auto upto = [&](int s) { return s < smin ? 0 : s >= smax ? N : __ldg(pre + (s - smin)); };
-  return hi < lo ? 0 : upto(hi) - upto(lo - 1);
-}
-
 __device__ int exact_coverage(const FastField& p, int x, int y, int av, int bv) {
   int c = 0;
   for (int i = 0; i < p.N; ++i) {
@@ -388,13 +333,6 @@ __device__ __forceinline__ Item decode_item(const FastField& ff, int f, int64_t 
   return it;
 }
 
-// Acquire a tensor map written to global memory before the launch for the
-// TMA unit (tensor-map proxy).
-__device__ __forceinline__ void tmap_acquire(const CUtensorMap* m) {
-  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"((uint64_t)m)
-               : "memory");
-}
-
 // Persistent kernel over every item of every field of the launch (BL:
 // bilinear sampling).  The last warp is the producer: it takes the next item from
 // the launch's work counter (dynamic, in the fields' longest-first order),
@@ -458,6 +396,7 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
   __shared__ int item_done[kItemSlots];     // consumer warps done with an item
   __shared__ Item item_info[kItemSlots];    // the items in flight
 
+  if (p.d_skip && *p.d_skip != 0) return;  // (uniform over the grid)
   T* smem = reinterpret_cast<T*>(reinterpret_cast<char*>(smem_raw) +
                                  ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1145,7 +1084,10 @@ struct Variant {
   int halves;  // x-velocity tiles per item (boxes per frame)
   int xpw;     // x-velocities per thread (2: a half holds two table tiles)
   const char* name;
+  bool runs = false;  // the run kernel (k_stack_runs.cu)
 };
+#define RUNS(T) \
+  {nullptr, nullptr, 0, 0, 16, 0, kTX, 4, 1, #T "_runs_ky8_x4_s3_f16", true}
 
 #define ST_VARIANT(T, KY, S, F, BL, CP, OPT, H)                                               \
   {                                                                                           \
@@ -1166,17 +1108,20 @@ struct Variant {
 #define ITEMXH(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, false, 48, 2)
 #define PAIR(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, true, 0, 1)
 #define BILI(T, KY, S, F) ST_VARIANT(T, KY, S, F, true, false, 0, 1)
-// (the first is the default; a two-velocity variant whose boxes do not hold
-// a field's motion runs as the first single-velocity one)
+// The last of each list is the default: the run kernel, which leaves the
+// fields that it does not take (motion beyond its boxes, a margin that is not
+// small against the noise, few frames) to the first or the third.  A two-velocity variant whose boxes
+// do not hold a field's motion runs as the first single-velocity one.
 const Variant kVarF32[] = {ITEMX(float, 8, 2, 16), ITEMH(float, 16, 2, 16), ITEM(float, 16, 2, 16),
                            ITEM(float, 16, 3, 12), ITEM(float, 16, 4, 8), ITEMH(float, 16, 4, 8),
                            NEAR(float, 16, 8, 4), NEAR(float, 24, 6, 4), PAIR(float, 8, 8, 4),
-                           ITEMXH(float, 8, 2, 16)};
+                           ITEMXH(float, 8, 2, 16), RUNS(float)};
 const Variant kVarF16[] = {ITEMX(__half, 8, 2, 16), ITEMH(__half, 16, 2, 16),
-                           ITEM(__half, 16, 2, 16), NEAR(__half, 16, 8, 4), PAIR(__half, 8, 8, 4)};
+                           ITEM(__half, 16, 2, 16), NEAR(__half, 16, 8, 4), PAIR(__half, 8, 8, 4),
+                           RUNS(__half)};
 const Variant kVarBF16[] = {ITEMX(__nv_bfloat16, 8, 2, 16), ITEMH(__nv_bfloat16, 16, 2, 16),
                             ITEM(__nv_bfloat16, 16, 2, 16), NEAR(__nv_bfloat16, 16, 8, 4),
-                            PAIR(__nv_bfloat16, 8, 8, 4)};
+                            PAIR(__nv_bfloat16, 8, 8, 4), RUNS(__nv_bfloat16)};
 // bilinear sampling: two window columns, one shared horizontal interpolation
 const Variant kVarBlF32[] = {BILI(float, 8, 8, 4), BILI(float, 12, 8, 4), BILI(float, 16, 6, 4)};
 const Variant kVarBlF16[] = {BILI(__half, 8, 8, 4), BILI(__half, 12, 8, 4)};
@@ -1187,8 +1132,10 @@ const Variant kVarBlBF16[] = {BILI(__nv_bfloat16, 8, 8, 4), BILI(__nv_bfloat16, 
 #undef ITEMX
 #undef ITEMXH
 #undef PAIR
+#undef RUNS
 #undef BILI
 #undef ST_VARIANT
+constexpr int kOneVelocity = 2;  // in each list of nearest variants: one velocity, 8 warps
 constexpr int kNumVariants = sizeof(kVarF32) / sizeof(kVarF32[0]);  // the largest list
 
 #define ST_LIST(L)                            \
@@ -1269,6 +1216,9 @@ struct FastPlan {
   int encoded_boxh = 0;
   int encoded_boxw = 0;
   int variant = 0;         // index into the (storage type, sampling) variant list
+  int ran = -1;            // the variant of the last launch
+  bool chosen = false;     // the variant was asked for (or autotuned), not the default
+  RunPlan* run = nullptr;  // the run kernel's tables (nearest sampling)
   bool bl = false;         // bilinear sampling
   int64_t item_limit = 0;  // > 0: run only the first item_limit items (autotuning)
   int nA = 0, nB = 0, N = 0;
@@ -1332,12 +1282,14 @@ int fast_autotune(const FieldDev& fd, FastPlan* fp, int64_t items, Pending* pend
   fp->item_limit = items;
   for (int v = 0; v < n; ++v) {
     if (vars[v].xpw > 1 && !fp->fits_x2) continue;  // its boxes do not hold the motion
+    if (vars[v].runs && !(fp->run && fp->run->fits)) continue;
     fp->variant = v;
     float ms_min = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {  // first run warms up
       cudaEventRecord(e0, s);
-      int l = launch_stack_fast(fd, fp, 0, fd.nvx * fd.nvy, nullptr, nullptr, nullptr, pend,
-                                pend_cap, ctr, s);
+      RunCtl rc{};
+      rc.runs = true;
+      int l = launch_stack_fast_multi(&fd, &fp, 1, nullptr, nullptr, pend, pend_cap, ctr, &rc, s);
       cudaEventRecord(e1, s);
       if (l < 0 || cudaEventSynchronize(e1) != cudaSuccess) break;
       launches += l;
@@ -1359,13 +1311,14 @@ int fast_autotune(const FieldDev& fd, FastPlan* fp, int64_t items, Pending* pend
 const char* fast_variant_name(const FastPlan* fp, int storage) {
   int n = 0;
   const Variant* vars = variants_for(storage, fp && fp->bl, &n);
-  int v = fp ? fp->variant : -1;
-  if (v >= 0 && v < n && vars[v].xpw > 1 && !fp->fits_x2)
-    v = single_velocity_fallback(vars, n);  // as the launch runs it
+  const int v = fp ? fp->ran : -1;
   return v >= 0 && v < n ? vars[v].name : "?";
 }
 void fast_set_variant(FastPlan* fp, int v) {
-  if (fp && v >= 0 && v < kNumVariants) fp->variant = v;
+  if (fp && v >= 0 && v < kNumVariants) {
+    fp->variant = v;
+    fp->chosen = true;
+  }
 }
 
 bool fast_eligible(const FieldDev& fd, int mode) {
@@ -1382,6 +1335,9 @@ bool fast_plan_build(const FieldDev& fd, int mode, FastPlan** out) {
   fp->nB = (fd.nvy + kMB - 1) / kMB;
   fp->N = fd.N;
   fp->bl = mode == ST_BILINEAR;
+  int nvar = 0;
+  const Variant* vars = variants_for(fd.storage, fp->bl, &nvar);
+  fp->variant = vars[nvar - 1].runs ? nvar - 1 : 0;
   const size_t nfx = fp->bl ? (size_t)fd.N * fp->nA * kXV : 1;
   const size_t nfy = fp->bl ? (size_t)fd.N * fp->nB * kMB : 1;
   bool good = cudaMalloc(&fp->fxt, sizeof(float) * nfx) == cudaSuccess &&
@@ -1393,6 +1349,10 @@ bool fast_plan_build(const FieldDev& fd, int mode, FastPlan** out) {
               cudaMalloc(&fp->d_pat, (size_t)fd.N * fp->nB) == cudaSuccess &&
               cudaMalloc(&fp->d_ff, sizeof(FastField)) == cudaSuccess &&
               cudaMalloc(&fp->d_map, sizeof(CUtensorMap)) == cudaSuccess;
+  if (good && vars[nvar - 1].runs) {
+    fp->run = run_plan_build(fd, fp->nB);
+    good = fp->run != nullptr;
+  }
   if (!good) {
     fast_plan_free(fp);
     return false;
@@ -1413,6 +1373,7 @@ void fast_plan_free(FastPlan* fp) {
   cudaFree(fp->d_pat);
   cudaFree(fp->d_ff);
   cudaFree(fp->d_map);
+  run_plan_free(fp->run);
   delete fp;
 }
 
@@ -1446,7 +1407,9 @@ int fast_prepare(const FieldDev& fd, FastPlan* fp, cudaStream_t s, bool* fits) {
   k_shift_spread<<<(fd.nvx + 127) / 128, 128, 0, s>>>(fd.sx, fd.N, fd.nvx, maxes + 2);
   k_shift_spread<<<(fd.nvy + 127) / 128, 128, 0, s>>>(fd.sy, fd.N, fd.nvy, maxes + 2);
   cudaMemcpyAsync(fp->h_maxes, maxes, sizeof(int) * kMaxes, cudaMemcpyDeviceToHost, s);
+  if (fp->run) run_prepare(fd, fp->d_pat, fp->yt, nB, fp->run, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return 1;
+  if (fp->run) run_finish(fd, fp->run);
   // coverage prefix tables: one row per velocity, as long as the widest spread
   const int len = fp->h_maxes[2];
   const int64_t need = (int64_t)(fd.nvx + fd.nvy) * (len + 2);
@@ -1498,6 +1461,12 @@ int fast_prepare(const FieldDev& fd, FastPlan* fp, cudaStream_t s, bool* fits) {
   h.cov_xmax = cxmax;
   h.cov_ymin = cymin;
   h.cov_ymax = cymax;
+  if (fp->run) {
+    h.nG = fp->run->nG;
+    h.nT = fp->run->nT;
+    h.xg = fp->run->xg;
+    h.ord = fp->run->ord;
+  }
   if (cudaMemcpyAsync(fp->d_ff, &h, sizeof(FastField), cudaMemcpyHostToDevice, s) != cudaSuccess)
     return 1;
   // N >= 8 (two stages of 4 frames): the producer runs at most S stages (at
@@ -1515,35 +1484,91 @@ int fast_prepare(const FieldDev& fd, FastPlan* fp, cudaStream_t s, bool* fits) {
   return 1;
 }
 
-// The launch's variant (that of fps[0]) and, for every field, its cube's
-// tiled map for that variant's box, encoded and copied to the device when the
-// cube or the box changed (pageable source: staged before the call returns).
-static const Variant* stage_maps(const FieldDev* fds, FastPlan* const* fps, int n,
-                                 cudaStream_t s, bool* restaged, int* vi_out) {
+// Whether the run kernel takes these fields: their variant, motion within its
+// boxes and staircases, no dump.
+static bool runs_chosen(const FieldDev* fds, FastPlan* const* fps, int n) {
+  int nvar = 0;
+  const Variant* vars = variants_for(fds[0].storage, fps[0]->bl, &nvar);
+  const int v = fps[0]->variant;
+  if (v < 0 || v >= nvar || !vars[v].runs) return false;
+  double work = 0.0, many = 0.0;
+  int64_t items = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!fps[i]->run || !fps[i]->run->fits || fds[i].storage != fds[0].storage) return false;
+    const double w = (double)fds[i].W * fds[i].H * fds[i].N * fds[i].nvx * fds[i].nvy;
+    work += w;
+    if (fds[i].N >= 32) many += w;
+    items += run_items(fps[i]->h_ff);
+  }
+  // few frames: an item's runs are short and its end weighs more (512^2,
+  // 33^2 velocities, FP32: 8 frames 0.41 ms against 0.29 for the frame-order
+  // kernel, 24 frames 0.55 against 0.53, 64 frames 0.80 against 1.10)
+  // (nor where its items, of 32 x 32 pixels and 64 velocities, would not fill
+  // the SMs: 128^2 x 64, 9^2 velocities, 48 items 34 us against 28)
+  return fps[0]->chosen || (many >= 0.5 * work && items >= 152);
+}
+
+// The frame-order variant that the default stands for where the run kernel
+// does not take the fields: two x-velocities a thread, or, for short sequences
+// and where tiles of 16 x-velocities would pad the grid by more than a
+// twentieth, one (512^2, FP32: 33^2 velocities x 64 frames 1.28 against 1.10
+// ms; 2048^2 x 256, 801^2 velocities 0.61 against 0.58 of the FP32 pipe).
+// (its 16-row tiles bound an edge tile's coverage less closely and pass more
+// points on: a search whose pending list they overflow is done again without
+// `by_size`)
+static int plain_variant(const FieldDev* fds, FastPlan* const* fps, int n, bool by_size) {
+  int nvar = 0;
+  const Variant* vars = variants_for(fds[0].storage, fps[0]->bl, &nvar);
+  const int v = fps[0]->variant;
+  int vi = v >= 0 && v < nvar && !vars[v].runs ? v : 0;
+  if (by_size && v >= 0 && v < nvar && vars[v].runs) {
+    const int wide = (fds[0].nvx + 15) / 16 * 16, narrow = (fds[0].nvx + 7) / 8 * 8;
+    if (fds[0].N < 64 || 20 * wide > 21 * narrow) vi = kOneVelocity;
+  }
+  // a two-velocity variant needs every field's motion within its boxes
+  for (int i = 0; i < n && vars[vi].xpw > 1; ++i)
+    if (!fps[i]->fits_x2) vi = single_velocity_fallback(vars, nvar);
+  return vi;
+}
+
+bool fast_runs_chosen(const FieldDev* fds, FastPlan* const* fps, int n) {
+  return n >= 1 && runs_chosen(fds, fps, n);
+}
+
+// The variant (that of fps[0]; for the run kernel the one that stands in for
+// it) and, for every field, its cube's tiled map for that variant's box,
+// encoded and copied to the device when the cube or the box changed (pageable
+// source: staged before the call returns).  With `runs` the run kernel's maps
+// too.
+static const Variant* stage_maps(const FieldDev* fds, FastPlan* const* fps, int n, bool runs,
+                                 bool by_size, cudaStream_t s, bool* restaged, int* vi_out) {
   if (n < 1 || n > kMaxFields) return nullptr;
   FastPlan* fp0 = fps[0];
   int nvar = 0;
   const Variant* vars = variants_for(fds[0].storage, fp0->bl, &nvar);
-  int vi = fp0->variant < nvar ? fp0->variant : 0;
-  // a two-velocity variant needs every field's motion within its boxes
-  for (int i = 0; i < n && vars[vi].xpw > 1; ++i)
-    if (!fps[i]->fits_x2) vi = single_velocity_fallback(vars, nvar);
+  const int vi = plain_variant(fds, fps, n, by_size);
   const Variant& var = vars[vi];
   const int boxh = var.ky + 3 + (fp0->bl ? 1 : 0);
   const int boxw = box_w_of(var, fds[0].storage);
+  auto stage = [&](const FieldDev& fd, CUtensorMap* host, CUtensorMap* dev, int w, int h) {
+    if (!encode_tile_map(host, fd, w, h)) return false;
+    if (restaged) *restaged = true;
+    return cudaMemcpyAsync(dev, host, sizeof(CUtensorMap), cudaMemcpyHostToDevice, s) == cudaSuccess;
+  };
   for (int i = 0; i < n; ++i) {
     FastPlan* fp = fps[i];
     if (fds[i].storage != fds[0].storage || fp->bl != fp0->bl) return nullptr;
     if (fp->encoded_for != fds[i].cube || fp->encoded_boxh != boxh ||
         fp->encoded_boxw != boxw) {
-      if (!encode_tile_map(&fp->tmap, fds[i], boxw, boxh)) return nullptr;
-      if (cudaMemcpyAsync(fp->d_map, &fp->tmap, sizeof(CUtensorMap), cudaMemcpyHostToDevice,
-                          s) != cudaSuccess)
-        return nullptr;
+      if (!stage(fds[i], &fp->tmap, fp->d_map, boxw, boxh)) return nullptr;
       fp->encoded_for = fds[i].cube;
       fp->encoded_boxh = boxh;
       fp->encoded_boxw = boxw;
-      if (restaged) *restaged = true;
+    }
+    if (runs && fp->run->encoded_for != fds[i].cube) {
+      if (!stage(fds[i], &fp->run->tmap, fp->run->d_map, run_box_w(fds[i].storage), run_box_h()))
+        return nullptr;
+      fp->run->encoded_for = fds[i].cube;
     }
   }
   // kernel attributes are set once per compiled kernel
@@ -1566,26 +1591,65 @@ static const Variant* stage_maps(const FieldDev* fds, FastPlan* const* fps, int 
   return &var;
 }
 
-bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, cudaStream_t s,
+bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, bool plain, cudaStream_t s,
                 bool* restaged) {
   int vi = 0;
-  return stage_maps(fds, fps, n, s, restaged, &vi) != nullptr;
+  return stage_maps(fds, fps, n, !plain && runs_chosen(fds, fps, n), !plain, s, restaged, &vi) !=
+         nullptr;
+}
+
+void fast_note_ran(const FieldDev* fds, FastPlan* const* fps, int n, bool runs) {
+  const int vi = runs ? fps[0]->variant : plain_variant(fds, fps, n, true);
+  for (int i = 0; i < n; ++i) fps[i]->ran = vi;
 }
 
 int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, float* dump_S,
                             int32_t* dump_C, Pending* pend, int64_t pend_cap, Counters* ctr,
-                            cudaStream_t s) {
+                            const RunCtl* rc, cudaStream_t s) {
   FastPlan* fp0 = fps[0];  // the variant of the launch
+  const bool runs = rc && rc->runs && !dump_S && runs_chosen(fds, fps, n);
   int vi = 0;
-  const Variant* vp = stage_maps(fds, fps, n, s, nullptr, &vi);
+  const Variant* vp = stage_maps(fds, fps, n, runs, rc != nullptr, s, nullptr, &vi);
   if (!vp) return -1;
-  const Variant& var = *vp;
-  const int ky = var.ky, boxh = ky + 3 + (fp0->bl ? 1 : 0);
-  const int boxw = box_w_of(var, fds[0].storage);
   // fields longest first (the items of the most frames are taken first)
   int order[kMaxFields];
   for (int i = 0; i < n; ++i) order[i] = i;
   std::stable_sort(order, order + n, [&](int x, int y) { return fds[x].N > fds[y].N; });
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int launched = 0;
+  if (runs) {
+    thread_local static RunArgs r;
+    std::memset(&r, 0, sizeof r);
+    int64_t total = 0;
+    for (int i = 0; i < n; ++i) {
+      r.ff[i] = fps[order[i]]->d_ff;
+      r.maps[i] = fps[order[i]]->run->d_map;
+      r.margin[i] = rc->margin ? rc->margin[order[i]] : 0.0f;
+      total += run_items(fps[order[i]]->h_ff);
+    }
+    r.n_fields = n;
+    // (autotuning: 32 x 16 pixels and about 32 x-velocities an item)
+    const int64_t limit = (fp0->item_limit + 3) / 4;
+    r.n_items = limit > 0 && total > limit ? limit : total;
+    r.d_margin = rc->d_margin;
+    r.d_use = rc->d_use;
+    r.work = &ctr->work_next;
+    r.pend = pend;
+    r.cap = pend_cap;
+    r.ctr = ctr;
+    if (cudaMemsetAsync(&ctr->work_next, 0, sizeof(ctr->work_next), s) != cudaSuccess) return -1;
+    if (launch_runs(r, fds[0].storage, sms, s) < 0) return -1;
+    for (int i = 0; i < n; ++i) fps[i]->ran = fp0->variant;
+    launched = 1;
+    if (!rc->d_use) return launched;
+  } else {
+    for (int i = 0; i < n; ++i) fps[i]->ran = vi;
+  }
+  const Variant& var = *vp;
+  const int ky = var.ky, boxh = ky + 3 + (fp0->bl ? 1 : 0);
+  const int boxw = box_w_of(var, fds[0].storage);
   thread_local static FastArgs a;
   std::memset(&a, 0, sizeof a);
   int64_t total = 0;
@@ -1606,13 +1670,11 @@ int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, fl
   a.ctr = ctr;
   a.dump_S = dump_S;
   a.dump_C = dump_C;
+  a.d_skip = runs ? rc->d_use : nullptr;
   const int esz = fds[0].storage == ST_F32 ? 4 : 2;
   const int stage_bytes = ((boxh * boxw * esz) + 127) & ~127;
   void (*fn)(FastArgs) = dump_S ? var.dump_fn : var.fn;
   const size_t smem = (size_t)var.stages * var.halves * stage_bytes + 128;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (cudaMemsetAsync(&ctr->work_next, 0, sizeof(ctr->work_next), s) != cudaSuccess) return -1;
   // persistent CTAs per SM: as many as are resident at once (2 for KY <= 16),
   // queried once per compiled kernel
@@ -1629,7 +1691,7 @@ int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, fl
   if (cudaLaunchKernel((const void*)fn, dim3((unsigned)grid), dim3(var.threads), args, smem, s) !=
       cudaSuccess)
     return -1;
-  return 1;
+  return launched + 1;
 }
 
 int launch_stack_fast(const FieldDev& fd, const FastPlan* cfp, int k0, int nk,
@@ -1637,7 +1699,7 @@ int launch_stack_fast(const FieldDev& fd, const FastPlan* cfp, int k0, int nk,
                       int64_t pend_cap, Counters* ctr, cudaStream_t s) {
   if (k0 != 0 || nk != fd.nvx * fd.nvy || dump_k) return -1;  // whole grid only
   FastPlan* fp = const_cast<FastPlan*>(cfp);
-  return launch_stack_fast_multi(&fd, &fp, 1, dump_S, dump_C, pend, pend_cap, ctr, s);
+  return launch_stack_fast_multi(&fd, &fp, 1, dump_S, dump_C, pend, pend_cap, ctr, nullptr, s);
 }
 
 }  // namespace st

@@ -104,6 +104,9 @@ struct st_plan_s {
   int64_t link_ws_bytes = 0;
   int* d_rerr = nullptr;          // refinement timeout flag
   double* d_sky = nullptr;
+  unsigned* d_absmax = nullptr;   // per field: largest stored |value| (FP32 bits)
+  float* d_margin = nullptr;      // per field: margin of the run kernel
+  int* d_use = nullptr;           // whether the run kernel does the work
   st_candidate* d_hout = nullptr;
   int64_t hout_cap = 0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -159,6 +162,9 @@ void free_plan(st_plan_t* p) {
   cudaFree(p->d_tref);
   cudaFree(p->d_grid);
   cudaFree(p->d_sky);
+  cudaFree(p->d_absmax);
+  cudaFree(p->d_margin);
+  cudaFree(p->d_use);
   cudaFree(p->d_hout);
   if (p->e0) cudaEventDestroy(p->e0);
   if (p->e1) cudaEventDestroy(p->e1);
@@ -274,13 +280,15 @@ st_status prepare_tables(st_plan_t* p, int fi, const double* h_times, int64_t* l
   return ST_OK;
 }
 
-// Optional normalisation / storage conversion of field fi into the plan's cube.
-int64_t normalize_field(st_plan_t* p, int fi, const float* d_frames) {
+// Optional normalisation / storage conversion of field fi into the plan's cube
+// (largest: the largest stored value is wanted).
+int64_t normalize_field(st_plan_t* p, int fi, const float* d_frames, bool largest = false) {
   FieldPlan& fp = p->F[fi];
   fp.last_frames = d_frames;
   if (!fp.d_cube) return 0;
   return launch_normalize(d_frames, fp.f.n_frames, fp.P(), p->o.normalize, p->o.cr_clip,
-                          p->o.storage, fp.d_cube, nullptr, nullptr, p->d_sky, p->s);
+                          p->o.storage, fp.d_cube, nullptr, nullptr, p->d_sky,
+                          largest ? p->d_absmax + fi : nullptr, p->s);
 }
 
 // Tables + optional normalisation for field fi with the given frames/times.
@@ -314,8 +322,11 @@ FieldDev field_dev(const FieldPlan& fp, const float* d_frames, int fi, int stora
   return d;
 }
 
+// plain: with the default kernel that passes on the fewest points (the pending
+// list overflowed).
 st_status device_search(st_plan_t* p, const float* const* d_frames, const double* const* h_times,
-                        st_candidate* d_out, int64_t capacity, int64_t* h_count) {
+                        st_candidate* d_out, int64_t capacity, int64_t* h_count,
+                        bool plain = false) {
   if (!d_frames || !h_times || !h_count) return fail(ST_ERR_INVALID, "NULL argument");
   if (capacity < 0 || (capacity > 0 && !d_out))
     return fail(ST_ERR_INVALID, "capacity must be >= 0 and d_out non-NULL when capacity > 0");
@@ -385,13 +396,37 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
         std::swap(fast_fps[0], fast_fps[i]);
       }
     bool restaged = false;
-    if (!fast_stage(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(), p->s, &restaged)) {
+    if (!fast_stage(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(), plain, p->s,
+                    &restaged)) {
       for (int fi = 0; fi < nf; ++fi) use_fast[fi] = 0;  // every field: direct gather
       fast_fds.clear();
     }
     if (restaged) ++p->gen;
   }
   for (int fi = 0; fi < nf; ++fi) p->F[fi].last_variant = use_fast[fi] ? 1 : 0;
+
+  // The run kernel sums in another order than the plain definition and keeps
+  // points down to a margin below the threshold.  The margin follows from the
+  // largest value: the clip, where there is one; else it is found on the
+  // device, which then decides between the run kernel and the one that stands
+  // in for it.  (Unnormalised FP32 frames take a pass for it: as long as 40
+  // velocities' stacks, so grids of fewer than 256 leave it.)
+  bool runs = !plain && !fast_fds.empty() &&
+              fast_runs_chosen(fast_fds.data(), fast_fps.data(), (int)fast_fds.size());
+  const bool known = p->o.normalize && p->o.cr_clip > 0.0f;
+  std::vector<float> margin(fast_fds.size());
+  for (size_t i = 0; i < fast_fds.size() && runs; ++i) {
+    const FieldPlan& fp = p->F[fast_fds[i].field];
+    const double tau = fp.f.snr_threshold;
+    margin[i] = run_margin(1.01f * p->o.cr_clip, fp.f.n_frames,
+                           (float)(tau * std::sqrt((double)fp.f.n_frames)));
+    if (known)
+      runs = run_margin_ok(margin[i], fp.nmin, (float)(tau * std::sqrt((double)fp.nmin)));
+    else if (!fp.d_cube)
+      runs = fp.nk() >= 256;
+  }
+  const RunCtl rc{runs, known ? margin.data() : nullptr, known ? nullptr : p->d_margin,
+                  known ? nullptr : p->d_use};
 
   // ---- the device part of the search: normalise, stack, resolve, counters.
   // Errors are collected, not returned, so that a capture always ends.
@@ -403,13 +438,26 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   };
   auto issue = [&](int64_t* stack_launches, int64_t* launches) -> cudaError_t {
     cudaError_t e = cudaMemsetAsync(p->d_ctr, 0, sizeof(Counters), p->s);
-    for (int fi = 0; fi < nf; ++fi) *launches += normalize_field(p, fi, d_frames[fi]);
+    const bool largest = runs && !known;
+    if (largest && e == cudaSuccess)
+      e = cudaMemsetAsync(p->d_absmax, 0, sizeof(unsigned) * nf, p->s);
+    for (int fi = 0; fi < nf; ++fi) {
+      *launches += normalize_field(p, fi, d_frames[fi], largest && use_fast[fi]);
+      if (largest && use_fast[fi] && !p->F[fi].d_cube)
+        *launches += launch_absmax(d_frames[fi], p->F[fi].P() * p->F[fi].f.n_frames,
+                                   p->d_absmax + fi, p->s);
+    }
+    if (largest)
+      *launches += launch_run_margins(p->d_fds, nf, p->d_absmax, p->d_margin, p->d_use, p->s);
     if (e == cudaSuccess) e = record(p->e0);
     if (!fast_fds.empty()) {
       int n = launch_stack_fast_multi(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(),
-                                      nullptr, nullptr, p->d_pend, p->pend_cap, p->d_ctr, p->s);
+                                      nullptr, nullptr, p->d_pend, p->pend_cap, p->d_ctr,
+                                      plain ? nullptr : &rc, p->s);
       if (n < 0 && e == cudaSuccess) e = cudaErrorLaunchFailure;
-      *stack_launches += n > 0 ? n : 0;
+      // (of two launches one does the work, the other returns at once)
+      *stack_launches += n > 0 ? 1 : 0;
+      *launches += n > 1 ? n - 1 : 0;
     }
     for (int fi = 0; fi < nf; ++fi)
       if (!use_fast[fi])
@@ -427,7 +475,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   int64_t stack_launches = 0, dev_launches = 0;
   p->last_replayed = false;
   bool done = false;
-  if (p->o.use_graph && !p->graph_broken) {
+  if (p->o.use_graph && !p->graph_broken && !plain) {
     std::vector<const float*> key(d_frames, d_frames + nf);
     if (!(p->graph && p->graph_gen == p->gen && p->graph_frames == key)) {
       // capture the device part once for these frames and tables
@@ -488,6 +536,10 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   p->stack_ms = ms;
   p->stack_launches = stack_launches;
   Counters c = *p->h_ctr;
+  if (runs)
+    fast_note_ran(fast_fds.data(), fast_fps.data(), (int)fast_fps.size(), c.runs != 0);
+  if ((c.error & ERR_PENDING_OVERFLOW) && !plain && !fast_fds.empty())
+    return device_search(p, d_frames, h_times, d_out, capacity, h_count, true);
   if (c.error & ERR_PENDING_OVERFLOW) {
     *h_count = -1;
     p->launches = L;
@@ -635,6 +687,9 @@ st_status st_plan(const st_field* fields, int32_t n_fields, const st_opts* opts,
     guard(cudaMalloc(&p->d_grid, sizeof(double) * 4 * n_fields), "cudaMalloc(grid)");
     guard(cudaMalloc(&p->d_maps, sizeof(CUtensorMap) * n_fields), "cudaMalloc(maps)");
     guard(cudaMalloc(&p->d_rerr, sizeof(int)), "cudaMalloc(rerr)");
+    guard(cudaMalloc(&p->d_absmax, sizeof(unsigned) * n_fields), "cudaMalloc(absmax)");
+    guard(cudaMalloc(&p->d_margin, sizeof(float) * n_fields), "cudaMalloc(margin)");
+    guard(cudaMalloc(&p->d_use, sizeof(int)), "cudaMalloc(use)");
     if (st == ST_OK) {
       std::vector<double*> tp(n_fields);
       std::vector<double> tr(n_fields), gr(4 * n_fields);
@@ -742,7 +797,7 @@ st_status st_normalize(st_plan_t* p, int32_t field, const float* d_frames, void*
   double* d_ms = nullptr;
   CK(cudaMalloc(&d_ms, sizeof(double) * 2 * f.n_frames));
   launch_normalize(d_frames, f.n_frames, fp.P(), 1, p->o.cr_clip, p->o.storage, d_cube, d_ms,
-                   d_ms + f.n_frames, p->d_sky, p->s);
+                   d_ms + f.n_frames, p->d_sky, nullptr, p->s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && h_mu)
     e = cudaMemcpyAsync(h_mu, d_ms, sizeof(double) * f.n_frames, cudaMemcpyDeviceToHost, p->s);

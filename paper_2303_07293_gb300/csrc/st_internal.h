@@ -4,6 +4,7 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/st.h"
@@ -22,7 +23,7 @@ struct Counters {
   unsigned long long n_pending;   // points written (or attempted) to the pending list
   unsigned long long n_cand;      // candidates after the local-maximum test
   unsigned int error;             // bit flags, ERR_*
-  unsigned int pad;
+  unsigned int runs;              // 1: the run kernel did the stacking
   unsigned long long work_next;   // persistent-kernel work counter
 };
 
@@ -65,7 +66,33 @@ int launch_shift_tables(const double* d_t, int N, double t_ref, double vx0, doub
 size_t sky_partial_doubles(int N);
 int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float cr_clip,
                      int storage, void* cube, double* mu, double* sigma, double* partial,
-                     cudaStream_t s);
+                     unsigned* absmax, cudaStream_t s);
+// Largest |x| of n values that are not NaN, as FP32 bits, into *absmax (which
+// the caller zeroes; launch_normalize: of the stored values, if not NULL).
+int launch_absmax(const float* x, int64_t n, unsigned* absmax, cudaStream_t s);
+
+// Bound of the difference between the FP32 sum of N values of at most
+// `largest` in frame order and the run kernel's: an addition errs by at most
+// u = 2^-24 times its result.  Frame order: u largest (1 + 2 + .. + N).  Runs:
+// the running sums err as much (an output takes each frame from one of them,
+// and what two terms share of an earlier error cancels), and their terms, up
+// to 11 of at most N largest each, are added up in steps of at most 3 N
+// largest.  thr: the largest threshold, whose difference with the margin is
+// rounded too.
+__host__ __device__ inline float run_margin(float largest, int N, float thr) {
+  const float n = (float)N;
+  return 1.02f * 0x1p-24f * (largest * n * (n + 40.0f) + 4.0f * thr);
+}
+// Whether the margin is small against the noise of the least covered points:
+// the points it adds are then at most about a tenth of those above threshold.
+__host__ __device__ inline bool run_margin_ok(float margin, int nmin, float thr_nmin) {
+  const float root = sqrtf((float)(nmin > 1 ? nmin : 1));
+  const float tau = thr_nmin / root;
+  return margin * (tau > 1.0f ? tau : 1.0f) <= 0.1f * root;
+}
+// The margins of the n fields, and whether all are small, from the largest values.
+int launch_run_margins(const FieldDev* fds, int n, const unsigned* absmax, float* margin, int* use,
+                       cudaStream_t s);
 
 // Generic stack kernels over velocity indices [k0, k0+nk): threshold ->
 // pending list; optional dump of S and n_cov for the listed velocities.
@@ -99,11 +126,27 @@ int launch_stack_fast(const FieldDev& fd, const FastPlan* fp, int k0, int nk,
 // sampling; the variant of fps[0]), items taken longest field first.
 // Encodes and uploads the tensor maps a launch over these fields needs (so the
 // launch itself copies nothing); *restaged tells whether any map changed.
-bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, cudaStream_t s,
+// plain: for a launch without a RunCtl.
+bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, bool plain, cudaStream_t s,
                 bool* restaged);
+// Without `rc` the default variant is the frame-order kernel of 8-row tiles.
+// With it the default follows the field's sizes, and the run kernel may do the
+// work (k_stack_runs.cu): it keeps points
+// down to a margin below the threshold, given per field (margin, or d_margin in
+// device memory); with d_use it runs only if *d_use is not 0, else the
+// variant that stands in for it does (both are launched).
+struct RunCtl {
+  bool runs;              // the run kernel may do the work
+  const float* margin;    // host, [n] in the order of fds (NULL: 0)
+  const float* d_margin;  // device, by field of the plan
+  const int* d_use;
+};
+bool fast_runs_chosen(const FieldDev* fds, FastPlan* const* fps, int n);
+// Notes which of the two a launch with d_use ran (for the variant's name).
+void fast_note_ran(const FieldDev* fds, FastPlan* const* fps, int n, bool runs);
 int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, float* dump_S,
                             int32_t* dump_C, Pending* pend, int64_t pend_cap, Counters* ctr,
-                            cudaStream_t s);
+                            const RunCtl* rc, cudaStream_t s);
 
 // Local-maximum test of the pending points -> candidate list (unsorted) and keys.
 int launch_resolve(const FieldDev* fds_dev, int n_fields, int mode, const Pending* pend,
