@@ -17,7 +17,7 @@ namespace {
 template <typename T, int MODE>
 __device__ void stack_one(const FieldDev& fd, int x, int y, int a, int b, float& S, int& C) {
   const T* cube = (const T*)fd.cube;
-  const int64_t P = (int64_t)fd.W * fd.H;
+  const int64_t P = (int64_t)fd.pitch * fd.H;
   float acc = 0.0f;
   int cov = 0;
   for (int i = 0; i < fd.N; ++i) {
@@ -26,14 +26,16 @@ __device__ void stack_one(const FieldDev& fd, int x, int y, int a, int b, float&
     int w = y + __ldg(fd.sy + (int64_t)i * fd.nvy + b);
     if (MODE == ST_NEAREST) {
       bool in = u >= 0 && w >= 0 && u < fd.W && w < fd.H;
-      acc = __fadd_rn(acc, in ? load_px<T>(fr + (int64_t)w * fd.W + u) : 0.0f);
+      acc = __fadd_rn(acc, in ? load_px<T>(fr + (int64_t)w * fd.pitch + u) : 0.0f);
       cov += in;
     } else {
       float fx = __ldg(fd.fx + (int64_t)i * fd.nvx + a);
       float fy = __ldg(fd.fy + (int64_t)i * fd.nvy + b);
       BW wt = bilinear_weights(fx, fy);
-      acc = bilinear_acc(acc, wt, tap<T>(fr, fd.W, fd.H, u, w), tap<T>(fr, fd.W, fd.H, u + 1, w),
-                         tap<T>(fr, fd.W, fd.H, u, w + 1), tap<T>(fr, fd.W, fd.H, u + 1, w + 1));
+      acc = bilinear_acc(acc, wt, tap<T>(fr, fd.pitch, fd.W, fd.H, u, w),
+                         tap<T>(fr, fd.pitch, fd.W, fd.H, u + 1, w),
+                         tap<T>(fr, fd.pitch, fd.W, fd.H, u, w + 1),
+                         tap<T>(fr, fd.pitch, fd.W, fd.H, u + 1, w + 1));
       cov += bilinear_inside(u, fx, fd.W) && bilinear_inside(w, fy, fd.H);
     }
   }

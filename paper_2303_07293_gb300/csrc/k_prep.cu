@@ -542,13 +542,14 @@ __global__ void k_run_margins(const FieldDev* __restrict__ fds, int n,
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-    k_normalize_store(const float* __restrict__ raw, int64_t npix, int normalize, float cr_clip,
-                      const SkyState* __restrict__ state, T* __restrict__ cube,
+    k_normalize_store(const float* __restrict__ raw, int W, int H, int normalize, float cr_clip,
+                      const SkyState* __restrict__ state, T* __restrict__ cube, int pitch,
                       double* __restrict__ mu_out, double* __restrict__ sigma_out,
                       unsigned* __restrict__ absmax) {
   const int i = blockIdx.y;
+  const int64_t npix = (int64_t)W * H;
   const float* x = raw + (int64_t)i * npix;
-  T* o = cube + (int64_t)i * npix;
+  T* o = cube + (int64_t)i * pitch * H;
   // (one thread forms the frame's constants: FP64)
   __shared__ NormFrame s_f;
   if (normalize && threadIdx.x == 0) {
@@ -594,7 +595,7 @@ __global__ void __launch_bounds__(256)
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   // frames on 16-byte boundaries: four pixels a thread (one load, one store)
-  if (npix % 4 == 0 && ((reinterpret_cast<uintptr_t>(raw) & 15) | (reinterpret_cast<uintptr_t>(cube) & 15)) == 0) {
+  if (pitch == W && npix % 4 == 0 && ((reinterpret_cast<uintptr_t>(raw) & 15) | (reinterpret_cast<uintptr_t>(cube) & 15)) == 0) {
     for (int64_t j = first; j < npix / 4; j += stride) {
       const float4 r = __ldcs(reinterpret_cast<const float4*>(x) + j);
       const float4 w = values(r);
@@ -610,19 +611,26 @@ __global__ void __launch_bounds__(256)
     if (absmax) put_max(top, absmax);
     return;
   }
-  for (int64_t j = first; j < npix; j += 4 * stride) {
-    float4 r;
-    r.x = x[j];
-    r.y = j + stride < npix ? x[j + stride] : 0.0f;
-    r.z = j + 2 * stride < npix ? x[j + 2 * stride] : 0.0f;
-    r.w = j + 3 * stride < npix ? x[j + 3 * stride] : 0.0f;
-    r = values(r);
-    if (absmax)
-      top = fmaxf(top, fmaxf(fmaxf(fabsf(r.x), fabsf(r.y)), fmaxf(fabsf(r.z), fabsf(r.w))));
-    o[j] = to_store<T>(r.x);
-    if (j + stride < npix) o[j + stride] = to_store<T>(r.y);
-    if (j + 2 * stride < npix) o[j + 2 * stride] = to_store<T>(r.z);
-    if (j + 3 * stride < npix) o[j + 3 * stride] = to_store<T>(r.w);
+  // else a row a block, four strided pixels a thread
+  for (int y = blockIdx.x; y < H; y += gridDim.x) {
+    const float* xr = x + (int64_t)y * W;
+    T* orow = o + (int64_t)y * pitch;
+    for (int j = threadIdx.x; j < W; j += 1024) {
+      float4 r;
+      r.x = xr[j];
+      r.y = j + 256 < W ? xr[j + 256] : 0.0f;
+      r.z = j + 512 < W ? xr[j + 512] : 0.0f;
+      r.w = j + 768 < W ? xr[j + 768] : 0.0f;
+      r = values(r);
+      if (absmax)
+        top = fmaxf(top, fmaxf(fmaxf(fabsf(r.x), j + 256 < W ? fabsf(r.y) : 0.0f),
+                               fmaxf(j + 512 < W ? fabsf(r.z) : 0.0f,
+                                     j + 768 < W ? fabsf(r.w) : 0.0f)));
+      orow[j] = to_store<T>(r.x);
+      if (j + 256 < W) orow[j + 256] = to_store<T>(r.y);
+      if (j + 512 < W) orow[j + 512] = to_store<T>(r.z);
+      if (j + 768 < W) orow[j + 768] = to_store<T>(r.w);
+    }
   }
   if (absmax) put_max(top, absmax);
 }
@@ -644,9 +652,10 @@ size_t sky_partial_doubles(int N) {
   return (size_t)N * (kSkyBlocks * sizeof(SkyPartial) + sizeof(SkyState)) / sizeof(double);
 }
 
-int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float cr_clip,
-                     int storage, void* cube, double* mu, double* sigma, double* partial,
-                     unsigned* absmax, cudaStream_t s) {
+int launch_normalize(const float* raw, int N, int W, int H, int normalize, float cr_clip,
+                     int storage, void* cube, int pitch, double* mu, double* sigma,
+                     double* partial, unsigned* absmax, cudaStream_t s) {
+  const int64_t npix = (int64_t)W * H;
   int launches = 0;
   SkyPartial* parts = reinterpret_cast<SkyPartial*>(partial);
   SkyState* state = reinterpret_cast<SkyState*>(parts + (size_t)N * kSkyBlocks);
@@ -666,16 +675,16 @@ int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float
   dim3 g(bx, N);
   switch (storage) {
     case ST_F32:
-      k_normalize_store<float><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                 (float*)cube, mu, sigma, absmax);
+      k_normalize_store<float><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
+                                                 (float*)cube, pitch, mu, sigma, absmax);
       break;
     case ST_F16:
-      k_normalize_store<__half><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                  (__half*)cube, mu, sigma, absmax);
+      k_normalize_store<__half><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
+                                                  (__half*)cube, pitch, mu, sigma, absmax);
       break;
     default:
-      k_normalize_store<__nv_bfloat16><<<g, 256, 0, s>>>(raw, npix, normalize, cr_clip, state,
-                                                         (__nv_bfloat16*)cube, mu, sigma,
+      k_normalize_store<__nv_bfloat16><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
+                                                         (__nv_bfloat16*)cube, pitch, mu, sigma,
                                                          absmax);
       break;
   }

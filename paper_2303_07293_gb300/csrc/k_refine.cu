@@ -465,6 +465,8 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
   std::vector<CUtensorMap> maps(n_fields);
   int max_n = 0;
   for (int f = 0; f < n_fields; ++f) {
+    // (rows of the caller's frames, not of a padded copy)
+    if ((int64_t)h_fds[f].W * (h_fds[f].storage == ST_F32 ? 4 : 2) % 16 != 0) return -1;
     if (!encode_tile_map(&maps[f], h_fds[f], kBoxW, kBoxH)) return -1;
     max_n = h_fds[f].N > max_n ? h_fds[f].N : max_n;
   }

@@ -1246,9 +1246,9 @@ bool encode_tile_map(CUtensorMap* map, const FieldDev& fd, int box_w, int box_h)
   const CUtensorMapDataType dtype = fd.storage == ST_F32    ? Store<float>::kTma
                                     : fd.storage == ST_F16 ? Store<__half>::kTma
                                                            : Store<__nv_bfloat16>::kTma;
-  if (((int64_t)fd.W * esz) % 16 != 0) return false;  // row pitch: a multiple of 16 bytes
+  if (((int64_t)fd.pitch * esz) % 16 != 0) return false;  // row pitch: a multiple of 16 bytes
   cuuint64_t dims[3] = {(cuuint64_t)fd.W, (cuuint64_t)fd.H, (cuuint64_t)fd.N};
-  cuuint64_t strides[2] = {(cuuint64_t)fd.W * esz, (cuuint64_t)fd.W * fd.H * esz};
+  cuuint64_t strides[2] = {(cuuint64_t)fd.pitch * esz, (cuuint64_t)fd.pitch * fd.H * esz};
   cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_h, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return encode_fn()(map, dtype, 3, const_cast<void*>(fd.cube), dims, strides, box, estr,
@@ -1323,7 +1323,7 @@ void fast_set_variant(FastPlan* fp, int v) {
 
 bool fast_eligible(const FieldDev& fd, int mode) {
   const int align = fd.storage == ST_F32 ? 4 : 8;  // 16-byte rows for the tensor map
-  return (mode == ST_NEAREST || mode == ST_BILINEAR) && fd.W % align == 0 &&
+  return (mode == ST_NEAREST || mode == ST_BILINEAR) && fd.pitch % align == 0 &&
          encode_fn() != nullptr && fd.W >= 8 && fd.H >= 1;
 }
 

@@ -30,7 +30,8 @@ __global__ void __launch_bounds__(kTX* kTY)
   const int y = (tile / tiles_x) * kTY + (threadIdx.x >> 5);
   const bool pix_ok = x < W && y < H;
   const T* cube = (const T*)fd.cube;
-  const int64_t P = (int64_t)W * H;
+  const int pitch = fd.pitch;
+  const int64_t P = (int64_t)pitch * H, PO = (int64_t)W * H;  // a frame, an output plane
 
   int ka[kVG], kb[kVG], kidx[kVG];
   bool kok[kVG];
@@ -57,15 +58,16 @@ __global__ void __launch_bounds__(kTX* kTY)
       int u = x + sx, w = y + sy;
       if (MODE == ST_NEAREST) {
         bool in = u >= 0 && w >= 0 && u < W && w < H;
-        float s = in ? load_px<T>(fr + (int64_t)w * W + u) : 0.0f;
+        float s = in ? load_px<T>(fr + (int64_t)w * pitch + u) : 0.0f;
         acc[v] = __fadd_rn(acc[v], s);
         cov[v] += in;
       } else {
         float fx = __ldg(fd.fx + (int64_t)i * fd.nvx + ka[v]);
         float fy = __ldg(fd.fy + (int64_t)i * fd.nvy + kb[v]);
         BW wt = bilinear_weights(fx, fy);
-        acc[v] = bilinear_acc(acc[v], wt, tap<T>(fr, W, H, u, w), tap<T>(fr, W, H, u + 1, w),
-                              tap<T>(fr, W, H, u, w + 1), tap<T>(fr, W, H, u + 1, w + 1));
+        acc[v] = bilinear_acc(acc[v], wt, tap<T>(fr, pitch, W, H, u, w),
+                              tap<T>(fr, pitch, W, H, u + 1, w), tap<T>(fr, pitch, W, H, u, w + 1),
+                              tap<T>(fr, pitch, W, H, u + 1, w + 1));
         cov[v] += bilinear_inside(u, fx, W) && bilinear_inside(w, fy, H);
       }
     }
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(kTX* kTY)
     bool ok = pix_ok && kok[v];
     if (dump_S) {
       if (ok) {
-        int64_t o = (int64_t)(blockIdx.x * kVG + v) * P + (int64_t)y * W + x;
+        int64_t o = (int64_t)(blockIdx.x * kVG + v) * PO + (int64_t)y * W + x;
         dump_S[o] = acc[v];
         if (dump_C) dump_C[o] = cov[v];
       }

@@ -69,6 +69,8 @@ struct FieldPlan {
   float* d_thr = nullptr;
   float* d_rsq = nullptr;
   void* d_cube = nullptr;        // normalised / converted storage cube (owned)
+  int pitch = 0;                 // its row pitch: a multiple of 16 bytes
+  bool copied = false;           // it is a plain copy of the frames with that pitch
   float* d_frames_copy = nullptr; // device copy for the host-buffer entry point
   FastPlan* fast = nullptr;
   int last_variant = -1;
@@ -286,9 +288,9 @@ int64_t normalize_field(st_plan_t* p, int fi, const float* d_frames, bool larges
   FieldPlan& fp = p->F[fi];
   fp.last_frames = d_frames;
   if (!fp.d_cube) return 0;
-  return launch_normalize(d_frames, fp.f.n_frames, fp.P(), p->o.normalize, p->o.cr_clip,
-                          p->o.storage, fp.d_cube, nullptr, nullptr, p->d_sky,
-                          largest ? p->d_absmax + fi : nullptr, p->s);
+  return launch_normalize(d_frames, fp.f.n_frames, fp.f.width, fp.f.height, p->o.normalize,
+                          p->o.cr_clip, p->o.storage, fp.d_cube, fp.pitch, nullptr, nullptr,
+                          p->d_sky, largest ? p->d_absmax + fi : nullptr, p->s);
 }
 
 // Tables + optional normalisation for field fi with the given frames/times.
@@ -306,6 +308,7 @@ FieldDev field_dev(const FieldPlan& fp, const float* d_frames, int fi, int stora
   FieldDev d{};
   d.cube = fp.d_cube ? fp.d_cube : (const void*)d_frames;
   d.storage = fp.d_cube ? storage : ST_F32;
+  d.pitch = fp.d_cube ? fp.pitch : fp.f.width;
   d.W = fp.f.width;
   d.H = fp.f.height;
   d.N = fp.f.n_frames;
@@ -343,7 +346,6 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     if (st != ST_OK) return st;
     fds[fi] = field_dev(p->F[fi], d_frames[fi], fi, p->o.storage);
   }
-  CK(cudaMemcpyAsync(p->d_fds, fds.data(), sizeof(FieldDev) * nf, cudaMemcpyHostToDevice, p->s));
   // fields that fit the register-window kernel run in one persistent launch;
   // its variant is tuned (or looked up) on the field with the most work
   std::vector<char> use_fast(nf, 0);
@@ -360,6 +362,10 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
       fp.fast_ready = true;
     }
     use_fast[fi] = fp.fast && fp.fast_fits;
+    if (fp.copied && !use_fast[fi]) {  // the direct gather reads the frames as they are
+      fds[fi].cube = d_frames[fi];
+      fds[fi].pitch = fp.f.width;
+    }
     if (use_fast[fi]) {
       fast_fds.push_back(fds[fi]);
       fast_fps.push_back(fp.fast);
@@ -369,6 +375,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
         tune_fi = fi;
     }
   }
+  CK(cudaMemcpyAsync(p->d_fds, fds.data(), sizeof(FieldDev) * nf, cudaMemcpyHostToDevice, p->s));
   if (tune_fi >= 0 && p->o.tile == -1) {
     FieldPlan& tp = p->F[tune_fi];
     if (!tp.tuned) {
@@ -442,8 +449,11 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     if (largest && e == cudaSuccess)
       e = cudaMemsetAsync(p->d_absmax, 0, sizeof(unsigned) * nf, p->s);
     for (int fi = 0; fi < nf; ++fi) {
-      *launches += normalize_field(p, fi, d_frames[fi], largest && use_fast[fi]);
-      if (largest && use_fast[fi] && !p->F[fi].d_cube)
+      if (fds[fi].cube == d_frames[fi])
+        p->F[fi].last_frames = d_frames[fi];
+      else
+        *launches += normalize_field(p, fi, d_frames[fi], largest && use_fast[fi]);
+      if (largest && use_fast[fi] && fds[fi].cube == d_frames[fi])
         *launches += launch_absmax(d_frames[fi], p->F[fi].P() * p->F[fi].f.n_frames,
                                    p->d_absmax + fi, p->s);
     }
@@ -662,9 +672,25 @@ st_status st_plan(const st_field* fields, int32_t n_fields, const st_opts* opts,
     if (guard(cudaMalloc(&fp.d_rsq, sizeof(float) * (f.n_frames + 1)), "cudaMalloc(rsq)"))
       guard(cudaMemcpy(fp.d_rsq, rsq.data(), sizeof(float) * rsq.size(), cudaMemcpyHostToDevice),
             "cudaMemcpy(rsq)");
-    if (opts->normalize || opts->storage != ST_F32)
-      guard(cudaMalloc(&fp.d_cube, store_bytes(opts->storage) * (size_t)f.n_frames * fp.P()),
-            "cudaMalloc(cube)");
+    // rows of the plan's own cube start 16 bytes apart, as the tensor maps of
+    // the register-window kernels need (1021 x 997 x 45, BF16, 41^2
+    // velocities: the direct gather of unpadded rows took 72 ms, the stack
+    // kernels 4)
+    const int align = opts->storage == ST_F32 ? 4 : 8;
+    fp.pitch = (f.width + align - 1) / align * align;
+    const size_t cube_bytes =
+        store_bytes(opts->storage) * (size_t)f.n_frames * fp.pitch * (size_t)f.height;
+    if (opts->normalize || opts->storage != ST_F32) {
+      guard(cudaMalloc(&fp.d_cube, cube_bytes), "cudaMalloc(cube)");
+    } else if (fp.pitch != f.width && opts->tile != 1 && fp.nk() >= 128 && f.n_frames >= 8) {
+      // frames used as given, of another width: a padded copy, if it fits the
+      // memory and the grid repays it (a pass takes as long as about 40
+      // velocities' stacks)
+      if (cudaMalloc(&fp.d_cube, cube_bytes) == cudaSuccess)
+        fp.copied = true;
+      else
+        cudaGetLastError();
+    }
     if (st == ST_OK && opts->tile != 1) {
       FieldDev probe = field_dev(fp, nullptr, i, opts->storage);
       if (fast_eligible(probe, opts->mode) && !fast_plan_build(probe, opts->mode, &fp.fast))
@@ -796,8 +822,8 @@ st_status st_normalize(st_plan_t* p, int32_t field, const float* d_frames, void*
   const st_field& f = fp.f;
   double* d_ms = nullptr;
   CK(cudaMalloc(&d_ms, sizeof(double) * 2 * f.n_frames));
-  launch_normalize(d_frames, f.n_frames, fp.P(), 1, p->o.cr_clip, p->o.storage, d_cube, d_ms,
-                   d_ms + f.n_frames, p->d_sky, nullptr, p->s);
+  launch_normalize(d_frames, f.n_frames, f.width, f.height, 1, p->o.cr_clip, p->o.storage, d_cube,
+                   f.width, d_ms, d_ms + f.n_frames, p->d_sky, nullptr, p->s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && h_mu)
     e = cudaMemcpyAsync(h_mu, d_ms, sizeof(double) * f.n_frames, cudaMemcpyDeviceToHost, p->s);

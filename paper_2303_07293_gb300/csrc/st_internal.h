@@ -31,7 +31,8 @@ enum : unsigned { ERR_PENDING_OVERFLOW = 1u, ERR_CAND_OVERFLOW = 2u, ERR_TIMEOUT
 
 // Everything a kernel needs to read one field.  Plain data, passed by value.
 struct FieldDev {
-  const void* cube;      // storage cube [N][H][W] of `storage` type
+  const void* cube;      // storage cube [N][H][pitch] of `storage` type
+  int32_t pitch;         // elements from one row to the next (>= W)
   int32_t storage;       // st_dtype
   int32_t W, H, N;
   int32_t nvx, nvy;
@@ -64,9 +65,10 @@ int launch_shift_tables(const double* d_t, int N, double t_ref, double vx0, doub
 // Sky statistics (FP64, deterministic) and normalisation/conversion.
 //   partial: workspace of sky_partial_doubles(N) doubles.
 size_t sky_partial_doubles(int N);
-int launch_normalize(const float* raw, int N, int64_t npix, int normalize, float cr_clip,
-                     int storage, void* cube, double* mu, double* sigma, double* partial,
-                     unsigned* absmax, cudaStream_t s);
+//   cube: rows of W values, pitch values apart.
+int launch_normalize(const float* raw, int N, int W, int H, int normalize, float cr_clip,
+                     int storage, void* cube, int pitch, double* mu, double* sigma,
+                     double* partial, unsigned* absmax, cudaStream_t s);
 // Largest |x| of n values that are not NaN, as FP32 bits, into *absmax (which
 // the caller zeroes; launch_normalize: of the stored values, if not NULL).
 int launch_absmax(const float* x, int64_t n, unsigned* absmax, cudaStream_t s);
@@ -111,7 +113,7 @@ int fast_autotune(const FieldDev& fd, FastPlan* fp, int64_t items, Pending* pend
                   int64_t pend_cap, Counters* ctr, cudaStream_t s);
 const char* fast_variant_name(const FastPlan* fp, int storage);
 void fast_set_variant(FastPlan* fp, int v);
-// Whether the field can use the fast kernel at all (width a multiple of
+// Whether the field can use the fast kernel at all (row pitch a multiple of
 // 16 bytes for the tensor map).
 bool fast_eligible(const FieldDev& fd, int mode);
 // Builds the per-frame tile tables for the current shift tables; *fits tells

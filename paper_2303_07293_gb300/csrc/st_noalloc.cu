@@ -168,7 +168,7 @@ extern "C" st_status st_stack_search_noalloc(const st_field* field, int32_t mode
   FieldDev fd{};
   fd.cube = d_frames;
   fd.storage = ST_F32;
-  fd.W = f.width;
+  fd.W = fd.pitch = f.width;
   fd.H = f.height;
   fd.N = N;
   fd.nvx = f.nvx;

@@ -19,10 +19,10 @@ __device__ __forceinline__ float load_px<__nv_bfloat16>(const __nv_bfloat16* p) 
   return __bfloat162float(__ldg(p));
 }
 
-// Pixel (u, v) of a frame, 0 outside.
+// Pixel (u, v) of a frame whose rows are `pitch` apart, 0 outside.
 template <typename T>
-__device__ __forceinline__ float tap(const T* frame, int W, int H, int u, int v) {
-  return (u >= 0 && v >= 0 && u < W && v < H) ? load_px<T>(frame + (int64_t)v * W + u) : 0.0f;
+__device__ __forceinline__ float tap(const T* frame, int pitch, int W, int H, int u, int v) {
+  return (u >= 0 && v >= 0 && u < W && v < H) ? load_px<T>(frame + (int64_t)v * pitch + u) : 0.0f;
 }
 
 // Bilinear weights from the FP32 fractions: (1-fx)(1-fy), fx(1-fy), (1-fx)fy, fx fy,
