@@ -7,6 +7,8 @@
 // to later ones) needs neighbour stack values that the stack kernels never
 // store: they are recomputed here by the same ordered FP32 sum, so they are
 // bit-identical to the values the stack kernel formed.
+#include <algorithm>
+
 #include "st_internal.h"
 #include "st_sample.cuh"
 
@@ -14,104 +16,144 @@ namespace st {
 
 namespace {
 
+// Sums and coverage of the three pixels x - 1, x, x + 1 of a row, each in
+// frame order.  (y may lie outside the frame: every sample that does reads 0.)
 template <typename T, int MODE>
-__device__ void stack_one(const FieldDev& fd, int x, int y, int a, int b, float& S, int& C) {
+__device__ void stack_three(const FieldDev& fd, int x, int y, int a, int b, float (&S)[3],
+                            int (&C)[3]) {
   const T* cube = (const T*)fd.cube;
   const int64_t P = (int64_t)fd.pitch * fd.H;
-  float acc = 0.0f;
-  int cov = 0;
-  for (int i = 0; i < fd.N; ++i) {
+  const int W = fd.W, H = fd.H, pitch = fd.pitch, N = fd.N;
+  const int32_t* sx = fd.sx + a;
+  const int32_t* sy = fd.sy + b;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    S[q] = 0.0f;
+    C[q] = 0;
+  }
+#pragma unroll 4
+  for (int i = 0; i < N; ++i) {
     const T* fr = cube + (int64_t)i * P;
-    int u = x + __ldg(fd.sx + (int64_t)i * fd.nvx + a);
-    int w = y + __ldg(fd.sy + (int64_t)i * fd.nvy + b);
+    const int u = x + __ldg(sx + (int64_t)i * fd.nvx);
+    const int w = y + __ldg(sy + (int64_t)i * fd.nvy);
     if (MODE == ST_NEAREST) {
-      bool in = u >= 0 && w >= 0 && u < fd.W && w < fd.H;
-      acc = __fadd_rn(acc, in ? load_px<T>(fr + (int64_t)w * fd.pitch + u) : 0.0f);
-      cov += in;
+      const bool row = w >= 0 && w < H;
+      const T* r = fr + (int64_t)(row ? w : 0) * pitch;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const int uq = u + q - 1;
+        const bool in = row && uq >= 0 && uq < W;
+        S[q] = __fadd_rn(S[q], in ? load_px<T>(r + uq) : 0.0f);
+        C[q] += in;
+      }
     } else {
-      float fx = __ldg(fd.fx + (int64_t)i * fd.nvx + a);
-      float fy = __ldg(fd.fy + (int64_t)i * fd.nvy + b);
-      BW wt = bilinear_weights(fx, fy);
-      acc = bilinear_acc(acc, wt, tap<T>(fr, fd.pitch, fd.W, fd.H, u, w),
-                         tap<T>(fr, fd.pitch, fd.W, fd.H, u + 1, w),
-                         tap<T>(fr, fd.pitch, fd.W, fd.H, u, w + 1),
-                         tap<T>(fr, fd.pitch, fd.W, fd.H, u + 1, w + 1));
-      cov += bilinear_inside(u, fx, fd.W) && bilinear_inside(w, fy, fd.H);
+      const float fx = __ldg(fd.fx + (int64_t)i * fd.nvx + a);
+      const float fy = __ldg(fd.fy + (int64_t)i * fd.nvy + b);
+      const BW wt = bilinear_weights(fx, fy);
+      float t0[4], t1[4];  // taps of the row and of the one below
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        t0[q] = tap<T>(fr, pitch, W, H, u + q - 1, w);
+        t1[q] = tap<T>(fr, pitch, W, H, u + q - 1, w + 1);
+      }
+      const bool row = bilinear_inside(w, fy, H);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        S[q] = bilinear_acc(S[q], wt, t0[q], t0[q + 1], t1[q], t1[q + 1]);
+        C[q] += row && bilinear_inside(u + q - 1, fx, W);
+      }
     }
   }
-  S = acc;
-  C = cov;
 }
 
 template <int MODE>
-__device__ void stack_any(const FieldDev& fd, int x, int y, int a, int b, float& S, int& C) {
-  if (fd.storage == ST_F32) stack_one<float, MODE>(fd, x, y, a, b, S, C);
-  else if (fd.storage == ST_F16) stack_one<__half, MODE>(fd, x, y, a, b, S, C);
-  else stack_one<__nv_bfloat16, MODE>(fd, x, y, a, b, S, C);
+__device__ void stack_any(const FieldDev& fd, int x, int y, int a, int b, float (&S)[3],
+                          int (&C)[3]) {
+  if (fd.storage == ST_F32) stack_three<float, MODE>(fd, x, y, a, b, S, C);
+  else if (fd.storage == ST_F16) stack_three<__half, MODE>(fd, x, y, a, b, S, C);
+  else stack_three<__nv_bfloat16, MODE>(fd, x, y, a, b, S, C);
 }
 
-// 8 threads per pending point (one per neighbour), 32 points per block.
+// 4 lanes per pending point, of which three sum a row of three pixels each
+// (the row above, its own, the row below): the two shifts of a frame, which
+// are as many loads as a pixel's, serve three pixels, and the point's own sum
+// comes with its row.  2048^2 x 256, 101^2 velocities, 1 M points:
+// 8.2 ms (a neighbour a lane, the point itself after them: 22.1).
+// The grid is sized for the chip, not for the list's capacity (131 072 blocks
+// that found nothing to do took 76 us of a small search).
+constexpr int kResolveThreads = 256;
 template <int MODE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kResolveThreads)
     k_resolve(const FieldDev* __restrict__ fds, const Pending* __restrict__ pend,
               const Counters* __restrict__ ctr_in, int64_t pend_cap,
               st_candidate* __restrict__ cand, uint64_t* __restrict__ keys,
               uint32_t* __restrict__ idx, int64_t cand_cap, Counters* __restrict__ ctr) {
-  int64_t n = (int64_t)min((unsigned long long)pend_cap, ctr_in->n_pending);
-  int64_t p = (int64_t)blockIdx.x * 32 + (threadIdx.x >> 3);
-  int nb = threadIdx.x & 7;
-  int lane = threadIdx.x & 31;
-  bool have = p < n;
-  Pending r{};
-  bool q_in = false;
-  float Sq = 0.0f;
-  int Cq = 0;
-  int nmin = 0;
-  if (have) {
-    r = pend[p];
-    const FieldDev& fd = fds[r.field];
-    nmin = fd.nmin;
-    const int dxs[8] = {-1, 0, 1, -1, 1, -1, 0, 1};
-    const int dys[8] = {-1, -1, -1, 0, 0, 1, 1, 1};
-    int qx = r.x + dxs[nb], qy = r.y + dys[nb];
-    if (qx >= 0 && qy >= 0 && qx < fd.W && qy < fd.H) {
-      stack_any<MODE>(fd, qx, qy, r.k % fd.nvx, r.k / fd.nvx, Sq, Cq);
-      q_in = true;
-    }
-    // a point recorded by position only: its own sum and coverage, same order
-    if (nb == 0 && r.n_cov < 0) stack_any<MODE>(fd, r.x, r.y, r.k % fd.nvx, r.k / fd.nvx, r.S, r.n_cov);
-  }
-  const float Sc = __shfl_sync(0xffffffffu, r.S, lane & ~7);
-  const int Cc = __shfl_sync(0xffffffffu, r.n_cov, lane & ~7);
-  bool center_ok = false;
-  if (have) center_ok = Cc >= nmin && Sc >= __ldg(fds[r.field].thr + Cc);
-  const bool blocks = q_in && Cq >= nmin && (nb < 4 ? !(Sc > Sq) : !(Sc >= Sq));
-  unsigned bal = __ballot_sync(0xffffffffu, blocks);
-  unsigned group = (bal >> (lane & ~7)) & 0xffu;
-  bool is_cand = center_ok && nb == 0 && group == 0u;
-  unsigned m = __ballot_sync(0xffffffffu, is_cand);
-  if (m == 0u) return;
-  int leader = __ffs(m) - 1;
-  unsigned long long base = 0;
-  if (lane == leader) base = atomicAdd(&ctr->n_cand, (unsigned long long)__popc(m));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (is_cand) {
-    unsigned long long pos = base + __popc(m & ((1u << lane) - 1u));
-    if (pos < (unsigned long long)cand_cap) {
+  const int64_t n = (int64_t)min((unsigned long long)pend_cap, ctr_in->n_pending);
+  const int lane = threadIdx.x & 31, part = threadIdx.x & 3;
+  constexpr int kPoints = kResolveThreads / 4;
+  for (int64_t p0 = (int64_t)blockIdx.x * kPoints; p0 < n; p0 += (int64_t)gridDim.x * kPoints) {
+    const int64_t p = p0 + (threadIdx.x >> 2);
+    const bool have = p < n;
+    Pending r{};
+    float S[3] = {0.0f, 0.0f, 0.0f};
+    int C[3] = {0, 0, 0};
+    int nmin = 0, W = 0, H = 0;
+    if (have) {
+      r = pend[p];
       const FieldDev& fd = fds[r.field];
-      st_candidate c;
-      c.x = r.x;
-      c.y = r.y;
-      c.k = r.k;
-      c.field = r.field;
-      c.stack = r.S;
-      c.snr = __fmul_rn(r.S, __ldg(fd.rsq + r.n_cov));
-      c.n_cov = r.n_cov;
-      cand[pos] = c;
-      keys[pos] = cand_key(r.field, r.k, r.y, r.x);
-      idx[pos] = (uint32_t)pos;
-    } else {
-      atomicOr(&ctr->error, ERR_CAND_OVERFLOW);
+      nmin = fd.nmin;
+      W = fd.W;
+      H = fd.H;
+      const int y = r.y + part - 1;
+      if (part < 3 && y >= 0 && y < H)
+        stack_any<MODE>(fd, r.x, y, r.k % fd.nvx, r.k / fd.nvx, S, C);
+    }
+    // the point's own sum and coverage (recorded, or formed here)
+    float Sc = __shfl_sync(0xffffffffu, S[1], (lane & ~3) + 1);
+    int Cc = __shfl_sync(0xffffffffu, C[1], (lane & ~3) + 1);
+    if (r.n_cov >= 0) {
+      Sc = r.S;
+      Cc = r.n_cov;
+    }
+    const bool center_ok = have && Cc >= nmin && Sc >= __ldg(fds[r.field].thr + Cc);
+    // a neighbour inside the frame and covered blocks the point: earlier in
+    // raster order unless the point is greater, later unless it is at least equal
+    bool blocks = false;
+    const int y = r.y + part - 1;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int x = r.x + q - 1;
+      const bool other = part < 3 && !(part == 1 && q == 1);
+      const bool in = x >= 0 && x < W && y >= 0 && y < H && C[q] >= nmin;
+      const bool earlier = part == 0 || (part == 1 && q == 0);
+      blocks |= have && other && in && (earlier ? !(Sc > S[q]) : !(Sc >= S[q]));
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, blocks);
+    const bool is_cand = center_ok && part == 0 && ((bal >> (lane & ~3)) & 15u) == 0u;
+    const unsigned m = __ballot_sync(0xffffffffu, is_cand);
+    if (m == 0u) continue;
+    const int leader = __ffs(m) - 1;
+    unsigned long long base = 0;
+    if (lane == leader) base = atomicAdd(&ctr->n_cand, (unsigned long long)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (is_cand) {
+      const unsigned long long pos = base + __popc(m & ((1u << lane) - 1u));
+      if (pos < (unsigned long long)cand_cap) {
+        const FieldDev& fd = fds[r.field];
+        st_candidate c;
+        c.x = r.x;
+        c.y = r.y;
+        c.k = r.k;
+        c.field = r.field;
+        c.stack = Sc;
+        c.snr = __fmul_rn(Sc, __ldg(fd.rsq + Cc));
+        c.n_cov = Cc;
+        cand[pos] = c;
+        keys[pos] = cand_key(r.field, r.k, r.y, r.x);
+        idx[pos] = (uint32_t)pos;
+      } else {
+        atomicOr(&ctr->error, ERR_CAND_OVERFLOW);
+      }
     }
   }
 }
@@ -199,14 +241,14 @@ int launch_resolve(const FieldDev* fds_dev, int n_fields, int mode, const Pendin
                    const Counters* ctr, int64_t pend_cap, st_candidate* cand, uint64_t* keys,
                    uint32_t* idx, int64_t cand_cap, Counters* ctr_out, cudaStream_t s) {
   (void)n_fields;
-  // grid sized by the capacity; blocks past the live count exit at once
-  int64_t blocks = (pend_cap + 31) / 32;
+  const int64_t blocks = std::min((int64_t)8 * 152, (pend_cap + kResolveThreads / 4 - 1) /
+                                                        (kResolveThreads / 4));
   if (mode == ST_NEAREST)
-    k_resolve<ST_NEAREST><<<(unsigned)blocks, 256, 0, s>>>(fds_dev, pend, ctr, pend_cap, cand,
-                                                           keys, idx, cand_cap, ctr_out);
+    k_resolve<ST_NEAREST><<<(unsigned)blocks, kResolveThreads, 0, s>>>(
+        fds_dev, pend, ctr, pend_cap, cand, keys, idx, cand_cap, ctr_out);
   else
-    k_resolve<ST_BILINEAR><<<(unsigned)blocks, 256, 0, s>>>(fds_dev, pend, ctr, pend_cap, cand,
-                                                            keys, idx, cand_cap, ctr_out);
+    k_resolve<ST_BILINEAR><<<(unsigned)blocks, kResolveThreads, 0, s>>>(
+        fds_dev, pend, ctr, pend_cap, cand, keys, idx, cand_cap, ctr_out);
   return 1;
 }
 
