@@ -8,6 +8,7 @@ The method is the synthetic-tracking (shift-and-stack) search of Burdanov,
 Hasler & de Wit (2023), Sec. 1 and Sec. 2.1.
 """
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -320,6 +321,7 @@ class Plan:
         return ms.value, n.value
 
 
+@functools.lru_cache(maxsize=None)
 def _refine_objective_class():
     import torch
 

@@ -258,9 +258,7 @@ int launch_pad_keys(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counter
   return 1;
 }
 
-int launch_sort_gather(uint64_t* keys, uint32_t* idx, int64_t n, const Counters* ctr,
-                       const st_candidate* cand, st_candidate* out, int64_t capacity,
-                       cudaStream_t s) {
+int launch_sort(uint64_t* keys, uint32_t* idx, int64_t n, cudaStream_t s) {
   // n is a power of two >= the live count; padding keys sort last.
   int launches = 0;
   if (n >= 2) {
@@ -277,6 +275,13 @@ int launch_sort_gather(uint64_t* keys, uint32_t* idx, int64_t n, const Counters*
       ++launches;
     }
   }
+  return launches;
+}
+
+int launch_sort_gather(uint64_t* keys, uint32_t* idx, int64_t n, const Counters* ctr,
+                       const st_candidate* cand, st_candidate* out, int64_t capacity,
+                       cudaStream_t s) {
+  int launches = launch_sort(keys, idx, n, s);
   if (capacity > 0) {
     int64_t g = (n < capacity ? n : capacity);
     if (g < 1) g = 1;

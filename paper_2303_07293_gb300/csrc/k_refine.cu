@@ -28,10 +28,22 @@
 // outside the image takes the place of bounds tests; the box x origin is
 // rounded down to 16 bytes and the remainder is an index offset).  Thread t
 // owns cutout column t%64 and its 16 rows (t/64)*16.., so a warp reads 32
-// consecutive words of a box row; it walks its rows with the horizontal
-// interpolation h = a0 + fx (a1 - a0) of the row below carried over, so each
-// tap row is read and interpolated once.  Reductions use a fixed-order block
-// tree.  Every wait is bounded in time.
+// consecutive words of a box row, and handles its rows in pairs (k, k + 8):
+// tap rows q and q + 8 are one register pair, so the differences d = a1 - a0,
+// the horizontal interpolations h = a0 + fx d, their steps e = h' - h and the
+// sums are paired FP32 operations; the slope along x, whose weights (1 - fy)
+// and fy are the frame's, is summed as <g, d> and <g, d'>.  A ninth warp forms a
+// frame's shift when it issues the copy and leaves the fractions beside it;
+// each consumer warp releases a slot by itself (a consumer that issues the
+// copies paces all others: 48 ms).  Reductions use a fixed-order block tree.  Every wait is
+// bounded in time.
+//
+// What bounds it: per frame and cutout 272 shared-memory wavefronts and 66
+// paired operations a warp on the FP32 pipe, which paired FMAs of three distinct
+// register pairs reach at 0.67 of its rate (measured: 85 against 127 for adds, in
+// operations per clock and SM): about 400 clocks of the 590 it takes.  Half the
+// rows copied, 3 or 5 stages or three CTAs an SM: the same time.  4096
+// candidates x 300 frames x 21 evaluations: 62.5 ms with scalar operations, 48.2.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -47,19 +59,23 @@ namespace st {
 namespace {
 
 constexpr int kCut = 64;        // cutout side
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;   // consumers: 8 warps
+constexpr int kBlock = kThreads + 32;  // and the warp that issues the copies
 constexpr int kPix = kCut * kCut / kThreads;  // 16 rows of one column per thread
+constexpr int kHalf = kPix / 2;               // row pairs (k, k + 8)
 constexpr int kSums = 11;
-constexpr int kBoxW = 72;       // footprint columns: 65 taps + up to 7 of alignment
 constexpr int kBoxH = kCut + 1; // footprint rows
 constexpr uint64_t kWaitNs = 2000000000ull;  // wait limit: 2 s of wall-clock time
 
 template <typename T>
 constexpr int stages_for() { return sizeof(T) == 4 ? 4 : 6; }
 template <typename T>
-constexpr int box_bytes() { return ((kBoxW * kBoxH * (int)sizeof(T)) + 127) & ~127; }
-template <typename T>
 constexpr int align_elems() { return 16 / (int)sizeof(T); }
+// footprint columns: 65 taps and up to 3 (7 for 16-bit types) of alignment
+template <typename T>
+constexpr int box_w() { return kCut + align_elems<T>(); }
+template <typename T>
+constexpr int box_bytes() { return ((box_w<T>() * kBoxH * (int)sizeof(T)) + 127) & ~127; }
 
 struct RefineArgs {
   const FieldDev* fds;          // device field descriptors
@@ -71,6 +87,7 @@ struct RefineArgs {
   const int32_t* field_in;      // [n]    (eval mode)
   const st_candidate* cand;     // [n]    (optimise mode)
   const double* grid;           // per field: vx0, dvx, vy0, dvy (optimise mode)
+  const uint32_t* order;        // the candidates in the order they are taken (or NULL)
   int64_t n;
   float inv2s2, inv_s2;
   int steps;
@@ -94,7 +111,8 @@ __device__ __forceinline__ float ld_s<__nv_bfloat16>(const __nv_bfloat16* p) {
   return __bfloat162float(*p);
 }
 
-// Fixed-order block reduction of kSums values; result valid in thread 0.
+// Fixed-order reduction of kSums values over the consumers; result valid in
+// thread 0.  (The issuing warp meets its two barriers.)
 __device__ void block_sum(float (&v)[kSums], float* sh) {
 #pragma unroll
   for (int k = 0; k < kSums; ++k)
@@ -214,18 +232,19 @@ __device__ void gauss_newton_step(float* th, const float (&s)[kSums], const floa
 }
 
 template <typename T, bool OPT>
-__global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
+__global__ void __launch_bounds__(kBlock, 2) k_refine(RefineArgs a) {
   constexpr int S = stages_for<T>();
   constexpr int kBox = box_bytes<T>();
-  constexpr int kAl = align_elems<T>();
+  constexpr int kAl = align_elems<T>(), kBoxW = box_w<T>();
   extern __shared__ __align__(128) unsigned char dsm_raw[];
   __shared__ __align__(8) uint64_t full[S];
+  __shared__ __align__(8) uint64_t empty[S];  // the warps that are done with a slot
+  __shared__ float4 s_frame[S];  // a slot's frame: fx, fy, dt, column offset in the box
   __shared__ float sh[(kThreads / 32) * kSums];
   __shared__ float th[5];
   __shared__ double s_t12[2];   // sum dt, sum dt^2 (Gauss-Newton)
-  __shared__ int s_ok;
   unsigned char* ring = dsm_raw + ((128u - (smem_u32(dsm_raw) & 127u)) & 127u);
-  const int64_t c = blockIdx.x;
+  const int64_t c = a.order ? (int64_t)a.order[blockIdx.x] : (int64_t)blockIdx.x;
   if (c >= a.n) return;
   int fi, cx, cy;
   if (OPT) {
@@ -250,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
     const double* t = a.times[fi];
     const double t_ref = a.t_ref[fi];
     double p1 = 0.0, p2 = 0.0;
-    for (int j = tid; j < N; j += kThreads) {
+    for (int j = tid; j < N; j += kBlock) {
       const double d = t[j] - t_ref;
       sdt[j] = (float)d;
       sdt_lo[j] = (float)(d - (double)(float)d);
@@ -263,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
         p1 += __shfl_down_sync(0xffffffffu, p1, d);
         p2 += __shfl_down_sync(0xffffffffu, p2, d);
       }
-      __shared__ double s_p[2 * (kThreads / 32)];
+      __shared__ double s_p[2 * (kBlock / 32)];
       if ((tid & 31) == 0) {
         s_p[2 * (tid >> 5)] = p1;
         s_p[2 * (tid >> 5) + 1] = p2;
@@ -271,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
       __syncthreads();
       if (tid == 0) {
         double a1 = 0.0, a2 = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
+        for (int w = 0; w < kBlock / 32; ++w) {
           a1 += s_p[2 * w];
           a2 += s_p[2 * w + 1];
         }
@@ -282,9 +301,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
   }
   if (tid == 0) {
     tma_prefetch_desc(map);
-    for (int s = 0; s < S; ++s) mbar_init(&full[s], 1);
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kThreads / 32);
+    }
     mbar_init_fence();
-    s_ok = 1;
     if (OPT) {
       const st_candidate cd = a.cand[c];
       const double* gr = a.grid + 4 * fi;
@@ -299,17 +320,41 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
   }
   __syncthreads();
 
-  // thread 0 stages frame i (sequence number q) into ring slot q % S
-  uint32_t q_issued = 0;  // (thread 0) sequence number after the last staged frame
-  auto issue = [&](int i, uint32_t q, float vx, float vy) {
-    q_issued = q + 1;
-    const Shift f = frame_shift(vx, vy, sdt[i], sdt_lo[i]);
-    const int cu0 = cx - kCut / 2 + f.ux, cv0 = cy - kCut / 2 + f.uy;
-    const int bx = cu0 & ~(kAl - 1);  // 16-byte aligned box origin (floor, also below 0)
-    const int slot = (int)(q % S);
-    mbar_arrive_expect_tx(&full[slot], (uint32_t)(kBoxW * kBoxH * sizeof(T)));
-    tma_load_3d(ring + (size_t)slot * kBox, map, bx, cv0, i, &full[slot]);
-  };
+  if (tid >= kThreads) {
+    // ---- the issuing warp: frame i (sequence number q over all evaluations)
+    // into ring slot q % S once every consumer warp has left the slot
+    const int steps = OPT ? a.steps : 0;
+    uint32_t q = 0;
+    bool ok = true;
+    for (int step = 0; step <= steps; ++step) {
+      const float vx = th[0], vy = th[1];
+      if (tid == kThreads)
+        for (int i = 0; i < N && ok; ++i, ++q) {
+          const int slot = (int)(q % S);
+          if (q >= (uint32_t)S && !mbar_wait(&empty[slot], (q / S - 1) & 1u, kWaitNs)) {
+            ok = false;  // the frames that are not issued end the consumers' waits
+            break;
+          }
+          const Shift f = frame_shift(vx, vy, sdt[i], sdt_lo[i]);
+          const int cu0 = cx - kCut / 2 + f.ux, cv0 = cy - kCut / 2 + f.uy;
+          const int bx = cu0 & ~(kAl - 1);  // 16-byte aligned box origin (floor, also below 0)
+          s_frame[slot] = make_float4(f.fx, f.fy, sdt[i], __int_as_float(cu0 - bx));
+          mbar_arrive_expect_tx(&full[slot], (uint32_t)(kBoxW * kBoxH * sizeof(T)));
+          tma_load_3d(ring + (size_t)slot * kBox, map, bx, cv0, i, &full[slot]);
+        }
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      __syncthreads();  // (the two barriers of block_sum)
+      __syncthreads();
+      __syncthreads();  // the new parameters
+    }
+    // after a wait that gave up: the copies already issued land (bounded)
+    // before exit; only the latest phase of each slot can be waited on
+    if (!ok && tid == kThreads)
+      for (uint32_t k = q > (uint32_t)S ? q - S : 0; k < q; ++k)
+        mbar_wait(&full[k % S], (k / S) & 1u, kWaitNs);
+    return;
+  }
 
   const int col = tid % kCut;
   const int row0 = (tid / kCut) * kPix;
@@ -321,71 +366,78 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
   uint32_t q0 = 0;  // frames staged before this evaluation
   bool ok = true;
   for (int step = 0; step <= steps && ok; ++step) {
-    const float vx = th[0], vy = th[1], x0 = th[2], y0 = th[3];
-    if (tid == 0)
-      for (int i = 0; i < S && i < N; ++i) issue(i, q0 + i, vx, vy);
-    float S_[kPix], g[kPix];
+    const float x0 = th[2], y0 = th[3];
+    float2 S2[kHalf], g2[kHalf];
     const float dx = fcol - x0;
-#pragma unroll
-    for (int k = 0; k < kPix; ++k) {
-      S_[k] = 0.0f;
+    auto weight = [&](int k) {
       const float dy = frow0 + (float)k - y0;
-      g[k] = expf(-(dx * dx + dy * dy) * a.inv2s2);
+      return expf(-(dx * dx + dy * dy) * a.inv2s2);
+    };
+#pragma unroll
+    for (int k = 0; k < kHalf; ++k) {
+      S2[k] = make_float2(0.0f, 0.0f);
+      g2[k] = make_float2(weight(k), weight(k + kHalf));
     }
     float dvx = 0.0f, dvy = 0.0f;
     for (int i = 0; i < N; ++i) {
       const uint32_t q = q0 + i;
       const int slot = (int)(q % S);
-      if (!mbar_wait(&full[slot], (q / S) & 1u, kWaitNs)) {
-        atomicOr(a.err, 1);
-        s_ok = 0;
-      }
-      const float dt = sdt[i];
-      const Shift f = frame_shift(vx, vy, dt, sdt_lo[i]);
-      const int cu0 = cx - kCut / 2 + f.ux;
+      ok = mbar_wait(&full[slot], (q / S) & 1u, kWaitNs);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;  // (the other warps' waits run out too)
+      const float4 fr = s_frame[slot];
       const T* box = reinterpret_cast<const T*>(ring + (size_t)slot * kBox) +
-                     (size_t)row0 * kBoxW + (cu0 - (cu0 & ~(kAl - 1))) + col;
-      float a0 = ld_s<T>(box), a1 = ld_s<T>(box + 1);
-      float dp = a1 - a0;        // a1 - a0 of the row above
-      float hp = a0 + f.fx * dp; // its horizontal interpolation (top)
-      float gdx = 0.0f, gdy = 0.0f;
+                     (size_t)row0 * kBoxW + __float_as_int(fr.w) + col;
+      const float2 fx2 = make_float2(fr.x, fr.x), fy2 = make_float2(fr.y, fr.y);
+      const float2 neg = make_float2(-1.0f, -1.0f);
+      // tap rows q and q + 8 of the column and its right neighbour
+      float2 hp, dp;
+      float2 ga = make_float2(0.0f, 0.0f), gb = ga, ge = ga;  // <g, d>, <g, d'>, <g, e>
 #pragma unroll
-      for (int k = 0; k < kPix; ++k) {
-        const T* r = box + (k + 1) * kBoxW;
-        const float b0 = ld_s<T>(r), b1 = ld_s<T>(r + 1);
-        const float d = b1 - b0;
-        const float h = b0 + f.fx * d;   // bottom
-        const float dh = h - hp;         // bot - top
-        S_[k] += hp + f.fy * dh;
-        gdx += g[k] * (dp + f.fy * (d - dp));  // (1-fy)(a1-a0) + fy(b1-b0)
-        gdy += g[k] * dh;
+      for (int k = 0; k <= kHalf; ++k) {
+        const T* r = box + k * kBoxW;
+        const T* r8 = r + kHalf * kBoxW;
+        const float2 b0 = make_float2(ld_s<T>(r), ld_s<T>(r8));
+        const float2 b1 = make_float2(ld_s<T>(r + 1), ld_s<T>(r8 + 1));
+        const float2 d = __ffma2_rn(b0, neg, b1);   // b1 - b0, exact product
+        const float2 h = __ffma2_rn(fx2, d, b0);
+        if (k > 0) {
+          const float2 e = __ffma2_rn(hp, neg, h);
+          S2[k - 1] = __fadd2_rn(S2[k - 1], __ffma2_rn(fy2, e, hp));
+          ga = __ffma2_rn(g2[k - 1], dp, ga);
+          gb = __ffma2_rn(g2[k - 1], d, gb);
+          ge = __ffma2_rn(g2[k - 1], e, ge);
+        }
         hp = h;
         dp = d;
       }
-      dvx += dt * gdx;
-      dvy += dt * gdy;
-      __syncthreads();  // every thread is done with the slot
-      if (!s_ok) {
-        ok = false;
-        break;
-      }
-      if (tid == 0 && i + S < N) issue(i + S, q + S, vx, vy);
+      __syncwarp();
+      if ((tid & 31) == 0) mbar_arrive(&empty[slot]);
+      const float va = ga.x + ga.y, vb = gb.x + gb.y;
+      dvx += fr.z * (va + fr.y * (vb - va));
+      dvy += fr.z * (ge.x + ge.y);
     }
-    if (!ok) break;
+    ok = __syncthreads_and(ok);
+    if (!ok) {
+      if (tid == 0) atomicOr(a.err, 1);
+      break;
+    }
     q0 += (uint32_t)N;
 #pragma unroll
     for (int k = 0; k < kSums; ++k) sums[k] = 0.0f;
 #pragma unroll
     for (int k = 0; k < kPix; ++k) {
       const float dy = frow0 + (float)k - y0;
-      const float gx = g[k] * dx * a.inv_s2;
-      const float gy = g[k] * dy * a.inv_s2;
-      sums[0] += g[k] * S_[k];
-      sums[1] += g[k] * g[k];
-      sums[2] += gx * S_[k];
-      sums[3] += gy * S_[k];
-      sums[4] += g[k] * gx;
-      sums[5] += g[k] * gy;
+      const float g = k < kHalf ? g2[k % kHalf].x : g2[k % kHalf].y;
+      const float Sk = k < kHalf ? S2[k % kHalf].x : S2[k % kHalf].y;
+      const float gx = g * dx * a.inv_s2;
+      const float gy = g * dy * a.inv_s2;
+      sums[0] += g * Sk;
+      sums[1] += g * g;
+      sums[2] += gx * Sk;
+      sums[3] += gy * Sk;
+      sums[4] += g * gx;
+      sums[5] += g * gy;
       sums[8] += gx * gx;
       sums[9] += gy * gy;
       sums[10] += gx * gy;
@@ -432,12 +484,21 @@ __global__ void __launch_bounds__(kThreads, 2) k_refine(RefineArgs a) {
     }
     __syncthreads();
   }
-  if (!ok && tid == 0) {
-    // a wait gave up: let the copies already issued land (bounded) before
-    // exit; only the latest phase of each slot can be waited on
-    for (uint32_t q = q_issued > (uint32_t)S ? q_issued - S : 0; q < q_issued; ++q)
-      mbar_wait(&full[q % S], (q / S) & 1u, kWaitNs);
+}
+
+// Key of a candidate for the order by place: field, band of 32 rows, column.
+__global__ void k_refine_keys(const st_candidate* __restrict__ cand, int64_t n, int64_t n_pow2,
+                              uint64_t* __restrict__ keys, uint32_t* __restrict__ idx) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_pow2) return;
+  uint64_t key = ~0ull;
+  if (i < n) {
+    const st_candidate c = cand[i];
+    key = (uint64_t)(uint32_t)c.field << 48 | (uint64_t)((uint32_t)c.y >> 5 & 0xfffu) << 24 |
+          ((uint32_t)c.x & 0xffffffu);
   }
+  keys[i] = key;
+  idx[i] = i < n ? (uint32_t)i : 0xffffffffu;
 }
 
 template <typename T, bool OPT>
@@ -459,7 +520,8 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
                   int storage, bool optimise, const float* theta, const int32_t* centre,
                   const int32_t* field, const st_candidate* cand, int64_t n, int steps,
                   int optimizer, float fwhm, float lr_pos, float lr_vel, float* J, float* snr,
-                  float* grad, st_refined* out, int* err, cudaStream_t s) {
+                  float* grad, st_refined* out, int* err, uint64_t* keys, uint32_t* idx,
+                  int64_t sort_cap, cudaStream_t s) {
   if (n <= 0) return 0;
   // tensor maps of the fields' cubes (box: the footprint of one frame)
   std::vector<CUtensorMap> maps(n_fields);
@@ -467,7 +529,8 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
   for (int f = 0; f < n_fields; ++f) {
     // (rows of the caller's frames, not of a padded copy)
     if ((int64_t)h_fds[f].W * (h_fds[f].storage == ST_F32 ? 4 : 2) % 16 != 0) return -1;
-    if (!encode_tile_map(&maps[f], h_fds[f], kBoxW, kBoxH)) return -1;
+    if (!encode_tile_map(&maps[f], h_fds[f],
+                         h_fds[f].storage == ST_F32 ? box_w<float>() : box_w<__half>(), kBoxH)) return -1;
     max_n = h_fds[f].N > max_n ? h_fds[f].N : max_n;
   }
   if (max_n > refine_max_frames()) return -1;
@@ -485,6 +548,17 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
   a.cand = cand;
   a.grid = grid;
   a.n = n;
+  // More candidates than run at once, taken in the order of their places: CTAs
+  // that run together share frame footprints in L2 (4096 candidates x 300
+  // frames x 21 evaluations: 57.3 -> 51.0 ms; the sort takes 30 us).
+  int launches = 1;
+  int64_t pow2 = 1;
+  while (pow2 < n) pow2 <<= 1;
+  if (cand && n > 304 && n * max_n * (steps + 1) > (1 << 20) && pow2 <= sort_cap) {
+    k_refine_keys<<<(unsigned)((pow2 + 255) / 256), 256, 0, s>>>(cand, n, pow2, keys, idx);
+    launches += 1 + launch_sort(keys, idx, pow2, s);
+    a.order = idx;
+  }
   const double sg = fwhm / (2.0 * 1.1774100225154747);  // 2 sqrt(2 ln 2)
   a.inv2s2 = (float)(1.0 / (2.0 * sg * sg));
   a.inv_s2 = (float)(1.0 / (sg * sg));
@@ -502,7 +576,7 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
   do {                                                                                       \
     set_smem_attr<T, O>();                                                                   \
     const size_t smem = (size_t)stages_for<T>() * box_bytes<T>() + dt_bytes + 128;           \
-    k_refine<T, O><<<(unsigned)n, kThreads, smem, s>>>(a);                                   \
+    k_refine<T, O><<<(unsigned)n, kBlock, smem, s>>>(a);                                   \
   } while (0)
   if (storage == ST_F32) {
     if (optimise) ST_REF(float, true); else ST_REF(float, false);
@@ -512,7 +586,7 @@ int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUte
     if (optimise) ST_REF(__nv_bfloat16, true); else ST_REF(__nv_bfloat16, false);
   }
 #undef ST_REF
-  return 1;
+  return launches;
 }
 
 }  // namespace st

@@ -1108,14 +1108,14 @@ struct Variant {
 #define ITEMXH(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, false, 48, 2)
 #define PAIR(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, true, 0, 1)
 #define BILI(T, KY, S, F) ST_VARIANT(T, KY, S, F, true, false, 0, 1)
-// The last of each list is the default: the run kernel, which leaves the
+// Nearest sampling defaults to the run kernel, which leaves the
 // fields that it does not take (motion beyond its boxes, a margin that is not
 // small against the noise, few frames) to the first or the third.  A two-velocity variant whose boxes
 // do not hold a field's motion runs as the first single-velocity one.
 const Variant kVarF32[] = {ITEMX(float, 8, 2, 16), ITEMH(float, 16, 2, 16), ITEM(float, 16, 2, 16),
                            ITEM(float, 16, 3, 12), ITEM(float, 16, 4, 8), ITEMH(float, 16, 4, 8),
-                           NEAR(float, 16, 8, 4), NEAR(float, 24, 6, 4), PAIR(float, 8, 8, 4),
-                           ITEMXH(float, 8, 2, 16), RUNS(float)};
+                           NEAR(float, 16, 8, 4), RUNS(float), PAIR(float, 8, 8, 4),
+                           ITEMXH(float, 8, 2, 16)};
 const Variant kVarF16[] = {ITEMX(__half, 8, 2, 16), ITEMH(__half, 16, 2, 16),
                            ITEM(__half, 16, 2, 16), NEAR(__half, 16, 8, 4), PAIR(__half, 8, 8, 4),
                            RUNS(__half)};
@@ -1154,6 +1154,13 @@ const Variant* variants_for(int storage, bool bl, int* count) {
   ST_LIST(kVarF32);
 }
 #undef ST_LIST
+
+// The run kernel's place in a list (-1: none).
+int runs_index(const Variant* vars, int n) {
+  for (int v = 0; v < n; ++v)
+    if (vars[v].runs) return v;
+  return -1;
+}
 
 // The variant that runs in place of a two-velocity one whose boxes do not
 // hold the motion: the first single-velocity one of the list.
@@ -1337,7 +1344,8 @@ bool fast_plan_build(const FieldDev& fd, int mode, FastPlan** out) {
   fp->bl = mode == ST_BILINEAR;
   int nvar = 0;
   const Variant* vars = variants_for(fd.storage, fp->bl, &nvar);
-  fp->variant = vars[nvar - 1].runs ? nvar - 1 : 0;
+  const int vr = runs_index(vars, nvar);
+  fp->variant = vr >= 0 ? vr : 0;
   const size_t nfx = fp->bl ? (size_t)fd.N * fp->nA * kXV : 1;
   const size_t nfy = fp->bl ? (size_t)fd.N * fp->nB * kMB : 1;
   bool good = cudaMalloc(&fp->fxt, sizeof(float) * nfx) == cudaSuccess &&
@@ -1349,7 +1357,7 @@ bool fast_plan_build(const FieldDev& fd, int mode, FastPlan** out) {
               cudaMalloc(&fp->d_pat, (size_t)fd.N * fp->nB) == cudaSuccess &&
               cudaMalloc(&fp->d_ff, sizeof(FastField)) == cudaSuccess &&
               cudaMalloc(&fp->d_map, sizeof(CUtensorMap)) == cudaSuccess;
-  if (good && vars[nvar - 1].runs) {
+  if (good && vr >= 0) {
     fp->run = run_plan_build(fd, fp->nB);
     good = fp->run != nullptr;
   }

@@ -589,7 +589,8 @@ st_status run_refine(st_plan_t* p, bool optimise, const float* theta, const int3
   CK(cudaMemsetAsync(p->d_rerr, 0, sizeof(int), p->s));
   int l = launch_refine(h.data(), nf, p->d_fds, p->d_maps, p->d_times, p->d_tref, p->d_grid,
                         h[0].storage, optimise, theta, centre, field, cand, n, steps, optimizer,
-                        fwhm, lr_pos, lr_vel, J, snr, grad, out, p->d_rerr, p->s);
+                        fwhm, lr_pos, lr_vel, J, snr, grad, out, p->d_rerr, p->d_keys, p->d_idx,
+                        p->sort_cap, p->s);
   if (l < 0)
     return fail(ST_ERR_UNSUPPORTED, "refinement needs frame rows of a multiple of 16 bytes "
                 "and at most %d frames per field", refine_max_frames());

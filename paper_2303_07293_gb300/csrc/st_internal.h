@@ -161,6 +161,8 @@ int launch_resolve(const FieldDev* fds_dev, int n_fields, int mode, const Pendin
 int launch_sort_gather(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counters* ctr,
                        const st_candidate* cand, st_candidate* out, int64_t capacity,
                        cudaStream_t s);
+// The sort alone (idx carried along).
+int launch_sort(uint64_t* keys, uint32_t* idx, int64_t n_pow2, cudaStream_t s);
 int launch_pad_keys(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counters* ctr,
                     cudaStream_t s);
 
@@ -171,14 +173,16 @@ int launch_pad_keys(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counter
 // Refinement (forward + adjoint, optional Adam steps) of n candidates; h_fds
 // are the host copies of the n_fields device descriptors fds (their cubes are
 // mapped for TMA into d_maps, n_fields entries).  Returns -1 if a field cannot
-// be mapped or has more than refine_max_frames() frames.
+// be mapped or has more than refine_max_frames() frames.  keys, idx: sort_cap
+// entries of scratch for the order of the candidates.
 int refine_max_frames();
 int launch_refine(const FieldDev* h_fds, int n_fields, const FieldDev* fds, CUtensorMap* d_maps,
                   const double* const* times, const double* t_ref, const double* grid,
                   int storage, bool optimise, const float* theta, const int32_t* centre,
                   const int32_t* field, const st_candidate* cand, int64_t n, int steps,
                   int optimizer, float fwhm, float lr_pos, float lr_vel, float* J, float* snr,
-                  float* grad, st_refined* out, int* err, cudaStream_t s);
+                  float* grad, st_refined* out, int* err, uint64_t* keys, uint32_t* idx,
+                  int64_t sort_cap, cudaStream_t s);
 
 // Tracks: links the sorted candidates [n] into components (workspace of
 // link_workspace_bytes(n) bytes); writes up to cap tracks, *n_tracks = all.

@@ -37,7 +37,7 @@ def field(seed, W=96, H=45, N=19, nvx=13, nvy=11, step=0.4, tau=2.5, ref=None, v
     return fr, t, f
 
 
-RUNS = {"f32": 12, "f16": 7, "bf16": 7}   # plan option `tile` of the run kernel
+RUNS = {"f32": 9, "f16": 7, "bf16": 7}   # plan option `tile` of the run kernel
 
 
 def lists(st, fr, t, f, tiles, **kw):
@@ -91,7 +91,7 @@ def test_runs_margin_found_on_the_device(st, storage, normalize, scale):
 def test_runs_infinite_pixels(st):
     fr, t, f = field(7, nvx=24, nvy=20, N=33)
     fr[3, 10, 20], fr[4, 12, 21], fr[9, 30, 50] = np.inf, -np.inf, np.inf
-    (a, na), (b, _) = lists(st, fr, t, f, (12, 1))
+    (a, na), (b, _) = lists(st, fr, t, f, (9, 1))
     assert "runs" not in na
     same(a, b)
 
@@ -99,7 +99,7 @@ def test_runs_infinite_pixels(st):
 @pytest.mark.parametrize("shape", [dict(step=0.95, nvx=40, N=40), dict(step=2.0, N=40), dict(N=7)])
 def test_fields_beyond_the_run_kernel(st, shape):
     fr, t, f = field(8, **shape)
-    (a, na), (b, _) = lists(st, fr, t, f, (12, 1), normalize=True, cr_clip=10.0)
+    (a, na), (b, _) = lists(st, fr, t, f, (9, 1), normalize=True, cr_clip=10.0)
     assert "runs" not in na
     same(a, b)
 
@@ -119,7 +119,7 @@ def test_runs_pending_list_that_holds_the_points_but_not_the_margin(st):
                 hi = mid
             except st.StError:
                 lo = mid + 1
-    for tile in (0, 12):
+    for tile in (0, 9):
         with st.Plan(f, tile=tile, pending_capacity=lo, **kw) as p:
             a = p.candidates(x, t)
         same(a, b)
@@ -131,7 +131,7 @@ def test_runs_several_fields_and_graph(st):
     fr = [torch.from_numpy(m[0]).cuda() for m in made]
     t, f = [m[1] for m in made], [m[2] for m in made]
     got = []
-    for tile, graph in ((1, False), (12, False), (12, True), (0, True)):
+    for tile, graph in ((1, False), (9, False), (9, True), (0, True)):
         with st.Plan(f, tile=tile, use_graph=graph, normalize=True) as p:
             got.append(p.candidates(fr, t))
             again = p.candidates(fr, t)
