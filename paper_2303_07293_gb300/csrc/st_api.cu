@@ -889,7 +889,9 @@ st_status st_link_tracks(st_plan_t* p, const st_candidate* d_cand, int64_t n, in
   if (n > 0x7fffffffll) return fail(ST_ERR_UNSUPPORTED, "at most 2^31 - 1 detections");
   if (!p->has_search) return fail(ST_ERR_INVALID, "st_link_tracks needs a prior st_stack_search");
   if (n == 0) return ST_OK;
-  const int64_t need = link_workspace_bytes(n);
+  int64_t velocities = 0;
+  for (const FieldPlan& fp : p->F) velocities += fp.nk();
+  const int64_t need = link_workspace_bytes(n, velocities);
   if (need > p->link_ws_bytes) {
     cudaFree(p->d_link_ws);
     p->d_link_ws = nullptr;
@@ -898,8 +900,10 @@ st_status st_link_tracks(st_plan_t* p, const st_candidate* d_cand, int64_t n, in
     p->link_ws_bytes = need;
   }
   int64_t nt = 0;
-  int l = launch_link_tracks(d_cand, n, p->d_fds, p->d_grid, r_xy, r_v, p->d_link_ws, d_tracks,
-                             capacity, &nt, p->s);
+  // (the pinned counters are free between searches)
+  int l = launch_link_tracks(d_cand, n, p->d_fds, (int)p->F.size(), velocities, p->d_grid, r_xy,
+                             r_v, p->d_link_ws, d_tracks, capacity,
+                             reinterpret_cast<int*>(p->h_ctr), &nt, p->s);
   CK(cudaGetLastError());
   if (l < 0) return fail(ST_ERR_CUDA, "track linking failed");
   p->launches = l;
