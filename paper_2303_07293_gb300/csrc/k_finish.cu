@@ -227,6 +227,44 @@ __global__ void __launch_bounds__(kLocal / 2)
     }
 }
 
+// The sort and gather of a short list (at most kLocal candidates; a longer one
+// is left alone) in one block, the padding in shared memory only.
+__global__ void __launch_bounds__(kLocal / 2)
+    k_sort_short(const uint64_t* __restrict__ keys, const Counters* __restrict__ ctr,
+                 const st_candidate* __restrict__ cand, st_candidate* __restrict__ out,
+                 int64_t capacity) {
+  __shared__ uint64_t sk[kLocal];
+  __shared__ uint16_t si[kLocal];
+  if (ctr->n_cand == 0 || ctr->n_cand > kLocal || ctr->error != 0u) return;
+  const int n = (int)ctr->n_cand;
+  int m = 2;
+  while (m < n) m <<= 1;
+  for (int t = threadIdx.x; t < m; t += blockDim.x) {
+    sk[t] = t < n ? keys[t] : ~0ull;
+    si[t] = (uint16_t)t;
+  }
+  __syncthreads();
+  for (int k = 2; k <= m; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int t = threadIdx.x; t < m; t += blockDim.x) {
+        const int l = t ^ j;
+        if (l > t) {
+          const uint64_t a = sk[t], b = sk[l];
+          if ((a > b) == ((t & k) == 0)) {
+            sk[t] = b;
+            sk[l] = a;
+            const uint16_t q = si[t];
+            si[t] = si[l];
+            si[l] = q;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  const int g = (int)min((int64_t)n, capacity);
+  for (int t = threadIdx.x; t < g; t += blockDim.x) out[t] = cand[si[t]];
+}
+
 __global__ void k_gather(const uint32_t* __restrict__ idx, const Counters* __restrict__ ctr,
                          const st_candidate* __restrict__ cand, st_candidate* __restrict__ out,
                          int64_t capacity) {
@@ -255,6 +293,13 @@ int launch_resolve(const FieldDev* fds_dev, int n_fields, int mode, const Pendin
 int launch_pad_keys(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counters* ctr,
                     cudaStream_t s) {
   k_pad_keys<<<(unsigned)((n_pow2 + 255) / 256), 256, 0, s>>>(keys, idx, n_pow2, ctr);
+  return 1;
+}
+
+int64_t sort_short_max() { return kLocal; }
+int launch_sort_short(const uint64_t* keys, const Counters* ctr, const st_candidate* cand,
+                      st_candidate* out, int64_t capacity, cudaStream_t s) {
+  k_sort_short<<<1, kLocal / 2, 0, s>>>(keys, ctr, cand, out, capacity);
   return 1;
 }
 

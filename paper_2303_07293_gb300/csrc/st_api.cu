@@ -98,6 +98,7 @@ struct st_plan_s {
   uint32_t* d_idx = nullptr;
   int64_t sort_cap = 0;
   FieldDev* d_fds = nullptr;
+  std::vector<FieldDev> h_fds;    // what d_fds holds
   double** d_times = nullptr;  // per field: device pointer to its timestamps
   double* d_tref = nullptr;    // per field
   double* d_grid = nullptr;    // per field: vx0, dvx, vy0, dvy
@@ -375,7 +376,13 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
         tune_fi = fi;
     }
   }
-  CK(cudaMemcpyAsync(p->d_fds, fds.data(), sizeof(FieldDev) * nf, cudaMemcpyHostToDevice, p->s));
+  // (descriptors as uploaded before are there)
+  if (p->h_fds.size() != (size_t)nf ||
+      std::memcmp(p->h_fds.data(), fds.data(), sizeof(FieldDev) * nf) != 0) {
+    p->h_fds.clear();
+    CK(cudaMemcpyAsync(p->d_fds, fds.data(), sizeof(FieldDev) * nf, cudaMemcpyHostToDevice, p->s));
+    p->h_fds = fds;
+  }
   if (tune_fi >= 0 && p->o.tile == -1) {
     FieldPlan& tp = p->F[tune_fi];
     if (!tp.tuned) {
@@ -540,6 +547,9 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     if (e != cudaSuccess) return fail(ST_ERR_CUDA, "search: %s", cudaGetErrorString(e));
   }
   L += stack_launches + dev_launches;
+  // a short list is sorted before its length is known here
+  L += launch_sort_short(p->d_keys, p->d_ctr, p->d_cand, d_out, capacity, p->s);
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(p->s));
   float ms = 0.0f;
   CK(cudaEventElapsedTime(&ms, p->e0, p->e1));
@@ -563,11 +573,13 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     return fail(ST_ERR_TIMEOUT, "stack kernel: a pipeline wait gave up after 2 s");
   }
   int64_t n = (int64_t)c.n_cand;
-  int64_t sn = pow2_at_least(std::max<int64_t>(n, 1));
-  L += launch_pad_keys(p->d_keys, p->d_idx, sn, p->d_ctr, p->s);
-  L += launch_sort_gather(p->d_keys, p->d_idx, sn, p->d_ctr, p->d_cand, d_out, capacity, p->s);
-  CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(p->s));
+  if (n > sort_short_max()) {
+    int64_t sn = pow2_at_least(n);
+    L += launch_pad_keys(p->d_keys, p->d_idx, sn, p->d_ctr, p->s);
+    L += launch_sort_gather(p->d_keys, p->d_idx, sn, p->d_ctr, p->d_cand, d_out, capacity, p->s);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(p->s));
+  }
   p->launches = L;
   p->has_search = true;
   *h_count = n;

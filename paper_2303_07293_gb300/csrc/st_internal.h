@@ -161,6 +161,11 @@ int launch_resolve(const FieldDev* fds_dev, int n_fields, int mode, const Pendin
 int launch_sort_gather(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counters* ctr,
                        const st_candidate* cand, st_candidate* out, int64_t capacity,
                        cudaStream_t s);
+// The same for at most sort_short_max() candidates, whose number the kernel
+// reads itself (others, and lists with an error, are left alone).
+int64_t sort_short_max();
+int launch_sort_short(const uint64_t* keys, const Counters* ctr, const st_candidate* cand,
+                      st_candidate* out, int64_t capacity, cudaStream_t s);
 // The sort alone (idx carried along).
 int launch_sort(uint64_t* keys, uint32_t* idx, int64_t n_pow2, cudaStream_t s);
 int launch_pad_keys(uint64_t* keys, uint32_t* idx, int64_t n_pow2, const Counters* ctr,

@@ -185,6 +185,7 @@ extern "C" st_status st_stack_search_noalloc(const st_field* field, int32_t mode
   NA_CK(cudaMemsetAsync(ctr, 0, sizeof(Counters), s));  // the previous call's counts remain
   launch_stack_generic(fd, mode, 0, f.nvx * f.nvy, nullptr, nullptr, nullptr, pend, cap, ctr, s);
   launch_resolve(fdev, 1, mode, pend, ctr, cap, cand, keys, idx, cap, ctr, s);
+  launch_sort_short(keys, ctr, cand, d_out, capacity, s);
   NA_CK(cudaGetLastError());
   Counters hc;
   NA_CK(cudaMemcpyAsync(&hc, ctr, sizeof hc, cudaMemcpyDeviceToHost, s));
@@ -195,12 +196,14 @@ extern "C" st_status st_stack_search_noalloc(const st_field* field, int32_t mode
                    "no-alloc scratch", (unsigned long long)hc.n_pending, (long long)cap);
   }
   int64_t n = (int64_t)hc.n_cand;
-  int64_t sn = 1;
-  while (sn < n) sn <<= 1;
-  launch_pad_keys(keys, idx, sn, ctr, s);
-  launch_sort_gather(keys, idx, sn, ctr, cand, d_out, capacity, s);
-  NA_CK(cudaGetLastError());
-  NA_CK(cudaStreamSynchronize(s));
+  if (n > sort_short_max()) {
+    int64_t sn = 1;
+    while (sn < n) sn <<= 1;
+    launch_pad_keys(keys, idx, sn, ctr, s);
+    launch_sort_gather(keys, idx, sn, ctr, cand, d_out, capacity, s);
+    NA_CK(cudaGetLastError());
+    NA_CK(cudaStreamSynchronize(s));
+  }
   *h_count = n;
   if (n > capacity)
     return na_fail(ST_ERR_OVERFLOW, "%lld candidates exceed capacity %lld", (long long)n,
