@@ -273,6 +273,89 @@ def item_loop_x2(ky, frames, row_bytes, stages, warps, dtype="f32", wait_ns=2000
     return L, n_acc
 
 
+# bilinear sampling (rows per thread, frames per stage, box row bytes, ring
+# stages, consumer warps, storage)
+ITEMS_BL = ((12, 16, 160, 2, 8, "f32"), (16, 16, 160, 2, 8, "f32"), (12, 16, 96, 2, 8, "f16"), (12, 16, 96, 2, 8, "bf16"),
+            (8, 16, 160, 2, 8, "f32"), (8, 16, 96, 2, 8, "f16"), (8, 16, 96, 2, 8, "bf16"))
+ELEM = {"f32": 4, "f16": 2, "bf16": 2}
+
+
+def load_pair(dtype, reg, q, kh, row_bytes, col):
+    """PTX of pair {reg} = (window row q, row q + kh) of column col (0: the
+    thread's, 1: its right neighbour)."""
+    ld, cvt = DTYPES[dtype]
+    L = []
+    for r, row in ((2 * col, q), (2 * col + 1, q + kh)):
+        L.append(ld.format(r=r, o=row * row_bytes + col * ELEM[dtype]))
+        if cvt:
+            L += cvt.format(r=r).split("\n")
+    return L + [f"mov.b64 {reg}, {{sv{2 * col}, sv{2 * col + 1}}};"]
+
+
+def pattern_body_bl(p, ky, row_bytes, dtype="f32"):
+    """Bilinear body of pattern p: pair q of the horizontal interpolation
+    H = A + fx (B - A) of the window columns A, B is formed once, and added
+    with weight 1 - fy_j to pair m = q - c_j of y-velocity j and with weight
+    fy_j to pair m = q - c_j - 1 (the sample's upper and lower row)."""
+    kh = ky // 2
+    L = []
+    for q in range(kh + 4):
+        use = [(j, q - pat_off(p, j) - low, low) for low in (0, 1) for j in range(4)
+               if 0 <= q - pat_off(p, j) - low < kh]
+        if not use:
+            continue
+        if q > 0:
+            L += load_pair(dtype, "sA", q, kh, row_bytes, 0) + \
+                load_pair(dtype, "sB", q, kh, row_bytes, 1)
+        L += ["sub.rn.f32x2 sB, sB, sA;", "fma.rn.f32x2 sH, sX, sB, sA;"]
+        for j, m, low in use:
+            a = j * kh + m
+            L.append(f"fma.rn.f32x2 %{a}, {'sF' if low else 'sG'}{j}, sH, %{a};")
+    return L
+
+
+def item_loop_bl(ky, frames, row_bytes, stages, warps, dtype="f32", wait_ns=2000000000):
+    """As item_loop, for bilinear sampling: beside the word, a frame has the
+    warp's x-fraction as a pair (8 bytes, a warp's frames in a row) and, for
+    the 4 y-velocities, the pairs (fy, fy), (1 - fy, 1 - fy) (64 bytes).  Two
+    operands more: the addresses of the warp's x-fractions and of the
+    y-weights in slot 0."""
+    kh = ky // 2
+    n_acc = 4 * kh
+    slot = n_acc
+    lb, xb, yb = n_acc + 6, n_acc + 9, n_acc + 10
+    single, _ = item_loop(ky, frames, row_bytes, stages, warps, dtype, wait_ns=wait_ns)
+    head, tail = single[:single.index("SLOOP:")], single[single.index("SNEXT:"):]
+    k = [i for i, ln in enumerate(head) if ln.startswith(".reg .f32 sv<")][0]
+    head[k] = ".reg .f32 sv<4>;"
+    for i, ln in enumerate(head):
+        if ln.startswith(".reg .b16 sh<"):
+            head[i] = ".reg .b16 sh<4>;"
+        elif ln.startswith(".reg .u32 su<"):
+            head[i] = ".reg .u32 su<4>;"
+        elif ln.startswith(".reg .b64 sW<"):
+            head[i] = ".reg .b64 sA, sB, sH, sX, sF<4>, sG<4>;"
+    head.insert(1, ".reg .u32 sxp, syp;")
+    k = head.index("ld.shared.u32 sw, [swp];")
+    head[k:k] = [f"mad.lo.u32 sxp, %{slot}, {warps * frames * 8}, %{xb};",
+                 f"mad.lo.u32 syp, %{slot}, {frames * 64}, %{yb};"]
+    k = tail.index("add.u32 swp, swp, 4;")
+    tail[k + 1:k + 1] = ["add.u32 sxp, sxp, 8;", "add.u32 syp, syp, 64;"]
+    L = head + ["SLOOP:", "and.b32 sa, sw, 16777215;", f"add.u32 sa, sa, %{lb};",
+                "shr.u32 sid, sw, 24;", "ld.shared.u32 snw, [swp+4];",
+                "ld.shared.b64 sX, [sxp];"]
+    # every pattern uses pair 0 and the weights
+    L += load_pair(dtype, "sA", 0, kh, row_bytes, 0) + load_pair(dtype, "sB", 0, kh, row_bytes, 1)
+    L += [f"ld.shared.v2.b64 {{sF{j}, sG{j}}}, [syp+{16 * j}];" for j in range(4)]
+    L += ["BTT: .branchtargets " + ", ".join(f"BT{p}" for p in range(16)) + ";",
+          "brx.idx.uni sid, BTT;"]
+    for p in range(N_PATTERNS):
+        L.append(f"BT{p}:")
+        L += pattern_body_bl(p, ky, row_bytes, dtype)
+        L.append("bra.uni SNEXT;")
+    return L + ["BT15:"] + tail, n_acc
+
+
 def render():
     out = ["// Generated by gen_bodies.py: the consumer loop of the register-window",
            "// stack kernel (pattern bodies entered by brx.idx).  Do not edit.",
@@ -290,6 +373,18 @@ def render():
         out.append(f"#define ST_ITEMX2_KY{ky}_F{frames}_R{row_bytes}_S{stages}_W{warps}{sfx} \\")
         for ln in lines:
             out.append(f'  "{ln}\\n\\t" \\')
+        out.append("")
+    for ky, frames, row_bytes, stages, warps, dtype in ITEMS_BL:
+        lines, n_acc = item_loop_bl(ky, frames, row_bytes, stages, warps, dtype)
+        out.append(f"#define ST_ITEMBL_KY{ky}_{dtype.upper()} \\")
+        for ln in lines:
+            out.append(f'  "{ln}\\n\\t" \\')
+        out.append("")
+    for ky in sorted({k[0] for k in ITEMS_BL}):
+        ops = ", ".join(f'"+l"(acc[{a}])' for a in range(4 * (ky // 2)))
+        out.append(f"#define ST_ITEMBL_OPERANDS_KY{ky}(acc, slot, ph, err, nst, skip, wb0, lb, fb0, eb0, xb, yb) \\")
+        out.append(f'  : {ops}, "+r"(slot), "+r"(ph), "=r"(err) \\')
+        out.append('  : "r"(nst), "r"(skip), "r"(wb0), "r"(lb), "r"(fb0), "r"(eb0), "r"(xb), "r"(yb) : "memory"')
         out.append("")
     for ky in sorted({k[0] for k in ITEMS}):
         n_acc = 4 * (ky // 2)

@@ -239,33 +239,18 @@ __device__ __forceinline__ void add_pattern_cp(float2 (&acc)[kMB][KY], const flo
     for (int r = 0; r < KY; ++r) acc[j][r] = __fadd2_rn(acc[j][r], w[r + pat_off(ID, j)]);
 }
 
-// Bilinear, factored: a warp's x-fraction is common to its 4 y-velocities, so
-// the horizontal interpolation h[r] = c0[r] + fx (c1[r] - c0[r]) of window row
-// r is formed once per frame and shared; y-velocity j then adds
-// (1 - fy_j) h[r + c_j] + fy_j h[r + c_j + 1] to output row r as two fused
-// multiply-adds, on row pairs (m, m + KY/2) as paired FMAs (fma.rn.f32x2)
-// with the pair window hp[q] = (h[q], h[q + KY/2]).  (The generic kernel
-// forms the same bilinear sample as four weighted taps; the two agree to
-// FP32 rounding, and the local-maximum resolver re-forms every reported
-// value with the generic arithmetic.)
-template <int KY, int C>
-__device__ __forceinline__ void add_bl_column(float2 (&acc)[KY / 2], float gy, float fy,
-                                              const float2 (&hp)[KY / 2 + 4]) {
-  const float2 g2 = make_float2(gy, gy), f2 = make_float2(fy, fy);
-#pragma unroll
-  for (int m = 0; m < KY / 2; ++m)
-    acc[m] = __ffma2_rn(f2, hp[m + C + 1], __ffma2_rn(g2, hp[m + C], acc[m]));
-}
-
-template <int KY, int ID>
-__device__ __forceinline__ void add_pattern_bl(float2 (&acc)[kMB][KY / 2], const float (&gy)[kMB],
-                                               const float (&fy)[kMB],
-                                               const float2 (&hp)[KY / 2 + 4]) {
-  add_bl_column<KY, pat_off(ID, 0)>(acc[0], gy[0], fy[0], hp);
-  add_bl_column<KY, pat_off(ID, 1)>(acc[1], gy[1], fy[1], hp);
-  add_bl_column<KY, pat_off(ID, 2)>(acc[2], gy[2], fy[2], hp);
-  add_bl_column<KY, pat_off(ID, 3)>(acc[3], gy[3], fy[3], hp);
-}
+// Bilinear sampling (generated loop only): a warp's x-fraction is common to
+// its 4 y-velocities, so the horizontal interpolation h[r] = c0[r] + fx (c1[r]
+// - c0[r]) of window row r is formed once per frame and shared; y-velocity j
+// then adds (1 - fy_j) h[r + c_j] + fy_j h[r + c_j + 1] to output row r as two
+// fused multiply-adds, on row pairs (m, m + KY/2) as paired FMAs
+// (fma.rn.f32x2).  (The generic kernel forms the same bilinear sample as four
+// weighted taps; the two agree to FP32 rounding, and the local-maximum
+// resolver re-forms every reported value with the generic arithmetic.)
+// 1024^2 x 64, 81^2 velocities: 63.5 ms with 12 rows a thread (68.3 with 8,
+// 67.5 with 16; a C++ switch on the pattern, whose FMAs the compiler left
+// unpaired: 84.5 with 8 rows, 76.4 with 12).  What bounds it: paired FMAs of
+// three distinct register pairs run at 0.67 of the pipe's rate.
 
 __device__ int exact_coverage(const FastField& p, int x, int y, int av, int bv) {
   int c = 0;
@@ -359,6 +344,7 @@ __device__ __forceinline__ Item decode_item(const FastField& ff, int f, int64_t 
 template <typename T, int KY, int S, int F, bool DUMP, bool BL, bool CP, int OPT, int H>
 __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
   static_assert(!(CP && BL), "column pairs are built for nearest sampling");
+  static_assert(!BL || (OPT & 16) != 0, "bilinear sampling runs in the generated item loop");
   static_assert(H == 1 || !(CP || BL), "two halves are built for single-column nearest sampling");
   constexpr bool kX2 = (OPT & 32) != 0;
   constexpr int kXPW = kX2 ? 2 : 1;        // x-velocities per thread
@@ -390,8 +376,10 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
   // the two windows' byte offsets, one unused), read as one vector
   constexpr int kWords = kX2 ? 4 : 1;
   __shared__ __align__(16) uint32_t slot_word[kLean ? S * kCW * F * kWords + 4 : 1];
-  __shared__ float slot_fx[BL ? S * F * kXV : 1];  // bilinear: x-fraction of each warp
-  __shared__ float4 slot_fy[BL ? S * F : 1];       // bilinear: y-fractions of the 4 y-velocities
+  // bilinear, as pairs of equal values: x-fraction of each warp, a warp's
+  // frames in a row; per frame and y-velocity (fy, fy, 1 - fy, 1 - fy)
+  __shared__ __align__(16) float slot_fx[BL ? S * F * kXV * 2 : 1];
+  __shared__ float4 slot_fy[BL ? S * F * kMB : 1];
   __shared__ int item_inside[kItemSlots * H];  // frames of an item half fully inside the frame
   __shared__ int item_done[kItemSlots];     // consumer warps done with an item
   __shared__ Item item_info[kItemSlots];    // the items in flight
@@ -588,10 +576,17 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
         const int fr = st * F + fi_l;
         if constexpr (!kLean) slot_ocol[(slot * H + h_l) * F + fi_l] = (uint32_t)cur.xe.y;
         if constexpr (BL) {
-          float* d = slot_fx + (slot * F + fi_l) * kXV;
-          d[0] = cur.f0.x; d[1] = cur.f0.y; d[2] = cur.f0.z; d[3] = cur.f0.w;
-          d[4] = cur.f1.x; d[5] = cur.f1.y; d[6] = cur.f1.z; d[7] = cur.f1.w;
-          slot_fy[slot * F + fi_l] = cur.fy;
+          const float fx8[kXV] = {cur.f0.x, cur.f0.y, cur.f0.z, cur.f0.w,
+                                  cur.f1.x, cur.f1.y, cur.f1.z, cur.f1.w};
+          float2* d = reinterpret_cast<float2*>(slot_fx) + slot * kXV * F + fi_l;
+#pragma unroll
+          for (int w = 0; w < kXV; ++w) d[w * F] = make_float2(fx8[w], fx8[w]);
+          const float fy4[kMB] = {cur.fy.x, cur.fy.y, cur.fy.z, cur.fy.w};
+#pragma unroll
+          for (int j = 0; j < kMB; ++j) {
+            const float gy = __fsub_rn(1.0f, fy4[j]);
+            slot_fy[(slot * F + fi_l) * kMB + j] = make_float4(fy4[j], fy4[j], gy, gy);
+          }
         }
         // every sample of the half strictly inside (bilinear: with its right
         // and lower taps), so every output of the half is covered
@@ -668,7 +663,7 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
 
     bool ok = true;
     if constexpr (kItemPtx) {
-      static_assert(KY == 16 || kX2, "the item loop is generated for KY = 16");
+      static_assert(KY == 16 || kX2 || BL, "the item loop is generated for KY = 16");
       constexpr bool kF32 = sizeof(T) == 4, kF16 = std::is_same<T, __half>::value;
       uint32_t slot = (uint32_t)c_slot, ph = c_ph, err = 0;
       __syncwarp();  // the item description is read before the block
@@ -678,6 +673,20 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
       const uint32_t nst = (uint32_t)spi, skip = 1u;
 #define ST_ITEM_ASM(NAME) \
   asm volatile(NAME ST_ITEM_OPERANDS_KY16(acc64, slot, ph, err, nst, skip, wb0, lb, fb0, eb0))
+      const uint32_t xb = smem_u32(&slot_fx[BL ? warp * F * 2 : 0]), yb = smem_u32(slot_fy);
+#define ST_ITEMBL_ASM(NAME, K)                                                             \
+  asm volatile(NAME ST_ITEMBL_OPERANDS_KY##K(acc64, slot, ph, err, nst, skip, wb0, lb, fb0, \
+                                             eb0, xb, yb))
+      if constexpr (BL) {
+        static_assert(!BL || (F == 16 && S == 2 && kCW == 8), "generated shape");
+        if constexpr (KY == 8 && kF32) ST_ITEMBL_ASM(ST_ITEMBL_KY8_F32, 8);
+        else if constexpr (KY == 8 && kF16) ST_ITEMBL_ASM(ST_ITEMBL_KY8_F16, 8);
+        else if constexpr (KY == 8) ST_ITEMBL_ASM(ST_ITEMBL_KY8_BF16, 8);
+        else if constexpr (KY == 16 && kF32) ST_ITEMBL_ASM(ST_ITEMBL_KY16_F32, 16);
+        else if constexpr (KY == 12 && kF32) ST_ITEMBL_ASM(ST_ITEMBL_KY12_F32, 12);
+        else if constexpr (KY == 12 && kF16) ST_ITEMBL_ASM(ST_ITEMBL_KY12_F16, 12);
+        else ST_ITEMBL_ASM(ST_ITEMBL_KY12_BF16, 12);
+      } else
       // (two x-velocities of 8 rows: 32 accumulator pairs, as 16 rows of one)
       if constexpr (kX2 && !kF32 && F == 16 && S == 2 && kCW == 8 && kF16)
         ST_ITEM_ASM(ST_ITEMX2_KY8_F16_R112_S2_W8_F16);
@@ -714,6 +723,7 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
       else
         static_assert(F == 0, "no generated item loop for these stages and warps");
 #undef ST_ITEM_ASM
+#undef ST_ITEMBL_ASM
       c_slot = (int)slot;
       c_ph = ph;
       if (err) {
@@ -751,45 +761,7 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
       for (int fi = 0; fi < F; ++fi) {
         const int id = (idw >> (8 * fi)) & 0xffu;
         const T* col = stage + fi * H * box_floats + ((ocw >> (4 * fi)) & 15u);
-        if constexpr (BL) {
-          float h[KY + 4];
-          const float fxw = slot_fx[(c_slot * F + fi) * kXV + xw];
-#pragma unroll
-          for (int r = 0; r < KY + 4; ++r) {
-            const float a0 = Store<T>::f(col[r * kBoxW]), a1 = Store<T>::f(col[r * kBoxW + 1]);
-            h[r] = __fmaf_rn(fxw, __fsub_rn(a1, a0), a0);
-          }
-          float2 hp[KY / 2 + 4];
-#pragma unroll
-          for (int q = 0; q < KY / 2 + 4; ++q) hp[q] = make_float2(h[q], h[q + KY / 2]);
-          const float4 fy4 = slot_fy[c_slot * F + fi];
-          if (fi == F - 1) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty_bar[c_slot]);
-          }
-          const float fy[kMB] = {fy4.x, fy4.y, fy4.z, fy4.w};
-          const float gy[kMB] = {__fsub_rn(1.0f, fy4.x), __fsub_rn(1.0f, fy4.y),
-                                 __fsub_rn(1.0f, fy4.z), __fsub_rn(1.0f, fy4.w)};
-          switch (id) {
-            case 0: add_pattern_bl<KY, 0>(acc, gy, fy, hp); break;
-            case 1: add_pattern_bl<KY, 1>(acc, gy, fy, hp); break;
-            case 2: add_pattern_bl<KY, 2>(acc, gy, fy, hp); break;
-            case 3: add_pattern_bl<KY, 3>(acc, gy, fy, hp); break;
-            case 4: add_pattern_bl<KY, 4>(acc, gy, fy, hp); break;
-            case 5: add_pattern_bl<KY, 5>(acc, gy, fy, hp); break;
-            case 6: add_pattern_bl<KY, 6>(acc, gy, fy, hp); break;
-            case 7: add_pattern_bl<KY, 7>(acc, gy, fy, hp); break;
-            case 8: add_pattern_bl<KY, 8>(acc, gy, fy, hp); break;
-            case 9: add_pattern_bl<KY, 9>(acc, gy, fy, hp); break;
-            case 10: add_pattern_bl<KY, 10>(acc, gy, fy, hp); break;
-            case 11: add_pattern_bl<KY, 11>(acc, gy, fy, hp); break;
-            case 12: add_pattern_bl<KY, 12>(acc, gy, fy, hp); break;
-            case 13: add_pattern_bl<KY, 13>(acc, gy, fy, hp); break;
-            case 14: add_pattern_bl<KY, 14>(acc, gy, fy, hp); break;
-            case kNoop: break;  // padding frame
-            default: __builtin_unreachable();
-          }
-        } else if constexpr (CP) {
+        if constexpr (CP) {
           float2 wp[KY + 3];  // rows of columns c and c + 32: register pairs
 #pragma unroll
           for (int r = 0; r < KY + 3; ++r)
@@ -1107,7 +1079,7 @@ struct Variant {
 #define ITEMX(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, false, 48, 1)
 #define ITEMXH(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, false, 48, 2)
 #define PAIR(T, KY, S, F) ST_VARIANT(T, KY, S, F, false, true, 0, 1)
-#define BILI(T, KY, S, F) ST_VARIANT(T, KY, S, F, true, false, 0, 1)
+#define BILX(T, KY, S, F) ST_VARIANT(T, KY, S, F, true, false, 16, 1)
 // Nearest sampling defaults to the run kernel, which leaves the
 // fields that it does not take (motion beyond its boxes, a margin that is not
 // small against the noise, few frames) to the first or the third.  A two-velocity variant whose boxes
@@ -1123,9 +1095,9 @@ const Variant kVarBF16[] = {ITEMX(__nv_bfloat16, 8, 2, 16), ITEMH(__nv_bfloat16,
                             ITEM(__nv_bfloat16, 16, 2, 16), NEAR(__nv_bfloat16, 16, 8, 4),
                             PAIR(__nv_bfloat16, 8, 8, 4), RUNS(__nv_bfloat16)};
 // bilinear sampling: two window columns, one shared horizontal interpolation
-const Variant kVarBlF32[] = {BILI(float, 8, 8, 4), BILI(float, 12, 8, 4), BILI(float, 16, 6, 4)};
-const Variant kVarBlF16[] = {BILI(__half, 8, 8, 4), BILI(__half, 12, 8, 4)};
-const Variant kVarBlBF16[] = {BILI(__nv_bfloat16, 8, 8, 4), BILI(__nv_bfloat16, 12, 8, 4)};
+const Variant kVarBlF32[] = {BILX(float, 12, 2, 16), BILX(float, 8, 2, 16), BILX(float, 16, 2, 16)};
+const Variant kVarBlF16[] = {BILX(__half, 12, 2, 16), BILX(__half, 8, 2, 16)};
+const Variant kVarBlBF16[] = {BILX(__nv_bfloat16, 12, 2, 16), BILX(__nv_bfloat16, 8, 2, 16)};
 #undef NEAR
 #undef ITEM
 #undef ITEMH
@@ -1133,7 +1105,7 @@ const Variant kVarBlBF16[] = {BILI(__nv_bfloat16, 8, 8, 4), BILI(__nv_bfloat16, 
 #undef ITEMXH
 #undef PAIR
 #undef RUNS
-#undef BILI
+#undef BILX
 #undef ST_VARIANT
 constexpr int kOneVelocity = 2;  // in each list of nearest variants: one velocity, 8 warps
 constexpr int kNumVariants = sizeof(kVarF32) / sizeof(kVarF32[0]);  // the largest list
