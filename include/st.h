@@ -101,7 +101,11 @@ typedef struct {
                                 window variant (tile - 2) of the list for the
                                 storage type and sampling (out of range: 0); a
                                 field whose motion does not fit the window takes
-                                the direct-gather kernel */
+                                the direct-gather kernel.  The default for
+                                nearest sampling adds frames with equal
+                                relative shifts once (the "runs" variant) and
+                                takes a frame-order variant for short fields;
+                                detections do not depend on the choice */
   const char* tune_cache;    /* JSON file for autotuned tiles, or NULL */
   int64_t pending_capacity;  /* above-threshold points held before the local-max
                                 test; 0 selects a default of 4 Mi points */
@@ -173,7 +177,9 @@ void st_free(st_plan_t* plan);
  * when the total exceeds capacity: the first `capacity` records of the sorted
  * list are written and *h_count holds the total, so a retry with a larger
  * buffer succeeds.  Returns ST_ERR_OVERFLOW with *h_count = -1 when the
- * above-threshold points exceed the plan's pending_capacity, and
+ * above-threshold points exceed the plan's pending_capacity (the default
+ * variant's filter is wider than the threshold by its rounding margin: if its
+ * points do not fit, the search is run again with a frame-order variant), and
  * ST_ERR_TIMEOUT (*h_count = -1) when a pipeline wait of the stack kernel
  * gave up after 2 s (the device stays usable).  Every field whose motion fits
  * the register-window kernel is searched in one persistent launch; shift
@@ -302,7 +308,8 @@ int32_t st_last_stack_variant(const st_plan_t* plan, int32_t field);
  * "direct-gather", the register-window variant's name (storage type, rows
  * per thread, ring stages, frames per stage, column pairs, code options:
  * o16 the generated item loop, o48 the same with two x-velocities a thread;
- * x-velocity tiles per block), or "?" before any search.  The string is
+ * x-velocity tiles per block; "runs" and the x-velocities of a group for the
+ * kernel that adds frames with equal relative shifts once), or "?" before any search.  The string is
  * static (owned by the library). */
 const char* st_stack_variant_name(const st_plan_t* plan, int32_t field);
 

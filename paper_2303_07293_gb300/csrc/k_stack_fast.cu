@@ -25,7 +25,7 @@
 //   the 4 y-velocities: y-velocity j reads window row r + c_j for output row
 //   r.  The row offsets c_j form a monotone staircase with steps of 0 or 1
 //   (15 patterns); the pattern is the same for the whole block in a frame, so
-//   one switch per frame picks a straight-line body.  Accumulators are held
+//   one indexed branch (or switch) per frame picks a straight-line body.  Accumulators are held
 //   as row pairs (m, m + KY/2) and the window as pairs (q, q + KY/2), so
 //   output pair m of y-velocity j adds window pair m + c_j: every add is a
 //   paired add (add.f32x2) whatever the offsets' parity (the column-pair
