@@ -502,9 +502,14 @@ __device__ __forceinline__ float normalize_pair(float r, const NormFrame& f, boo
   return none ? 0.0f : v;
 }
 
-// The warps' largest value into *absmax (values >= 0 order as their bits).
-__device__ __forceinline__ void put_max(float top, unsigned* absmax) {
-  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+// |v|'s bits, which order as the magnitudes do, an infinity above the finite
+// ones and a NaN above both: the run kernel's moves between running sums carry
+// either to outputs that never read the pixel, so both have to reach the margin.
+__device__ __forceinline__ unsigned mag(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+
+// The warps' largest magnitude into *absmax.
+__device__ __forceinline__ void put_max(unsigned top, unsigned* absmax) {
+  const unsigned m = __reduce_max_sync(0xffffffffu, top);
   if ((threadIdx.x & 31) == 0 && m > *absmax) atomicMax(absmax, m);
 }
 
@@ -513,15 +518,15 @@ __global__ void __launch_bounds__(256)
   const int64_t head = min(n, (int64_t)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15) / 4);
   const float4* v = reinterpret_cast<const float4*>(x + head);
   const int64_t nv = (n - head) / 4, tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float top = 0.0f;
-  if (tid < head) top = fabsf(x[tid]);
-  if (tid < n - head - 4 * nv) top = fmaxf(top, fabsf(x[head + 4 * nv + tid]));
+  unsigned top = 0u;
+  if (tid < head) top = mag(x[tid]);
+  if (tid < n - head - 4 * nv) top = max(top, mag(x[head + 4 * nv + tid]));
 #pragma unroll 4
   for (int64_t j = tid; j < nv; j += (int64_t)gridDim.x * blockDim.x) {
     const float4 q = __ldg(v + j);
-    top = fmaxf(top, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+    top = max(top, max(max(mag(q.x), mag(q.y)), max(mag(q.z), mag(q.w))));
   }
-  put_max(top > 0.0f ? top : 0.0f, absmax);  // (a NaN head or tail counts as 0)
+  put_max(top, absmax);
 }
 
 __global__ void k_run_margins(const FieldDev* __restrict__ fds, int n,
@@ -572,7 +577,7 @@ __global__ void __launch_bounds__(256)
   __syncthreads();
   const NormFrame f = s_f;
   auto clipped = [&](float v) { return cr_clip > 0.0f && fabsf(v) > cr_clip ? 0.0f : v; };
-  float top = 0.0f;
+  unsigned top = 0u;
   // four pixels; the FP64 formula sits behind one branch
   auto values = [&](float4 r) {
     if (!normalize) return r;
@@ -600,7 +605,7 @@ __global__ void __launch_bounds__(256)
       const float4 r = __ldcs(reinterpret_cast<const float4*>(x) + j);
       const float4 w = values(r);
       if (absmax)
-        top = fmaxf(top, fmaxf(fmaxf(fabsf(w.x), fabsf(w.y)), fmaxf(fabsf(w.z), fabsf(w.w))));
+        top = max(top, max(max(mag(w.x), mag(w.y)), max(mag(w.z), mag(w.w))));
       alignas(16) T v[4] = {to_store<T>(w.x), to_store<T>(w.y), to_store<T>(w.z),
                             to_store<T>(w.w)};
       if constexpr (sizeof(T) == 4)
@@ -623,9 +628,8 @@ __global__ void __launch_bounds__(256)
       r.w = j + 768 < W ? xr[j + 768] : 0.0f;
       r = values(r);
       if (absmax)
-        top = fmaxf(top, fmaxf(fmaxf(fabsf(r.x), j + 256 < W ? fabsf(r.y) : 0.0f),
-                               fmaxf(j + 512 < W ? fabsf(r.z) : 0.0f,
-                                     j + 768 < W ? fabsf(r.w) : 0.0f)));
+        top = max(top, max(max(mag(r.x), j + 256 < W ? mag(r.y) : 0u),
+                           max(j + 512 < W ? mag(r.z) : 0u, j + 768 < W ? mag(r.w) : 0u)));
       orow[j] = to_store<T>(r.x);
       if (j + 256 < W) orow[j + 256] = to_store<T>(r.y);
       if (j + 512 < W) orow[j + 512] = to_store<T>(r.z);

@@ -87,6 +87,7 @@ __host__ __device__ inline float run_margin(float largest, int N, float thr) {
 }
 // Whether the margin is small against the noise of the least covered points:
 // the points it adds are then at most about a tenth of those above threshold.
+// (False for a margin that an infinite or NaN value made.)
 __host__ __device__ inline bool run_margin_ok(float margin, int nmin, float thr_nmin) {
   const float root = sqrtf((float)(nmin > 1 ? nmin : 1));
   const float tau = thr_nmin / root;

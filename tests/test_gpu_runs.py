@@ -81,11 +81,28 @@ def test_runs_margin_found_on_the_device(st, storage, normalize, scale):
     # threshold is for leave the field to the other kernels
     fr, t, f = field(6, nvx=24, nvy=20, N=40)
     fr[3, 10, 20] = 30.0 * scale
-    fr[7, 11, 22] = np.nan
+    if normalize:   # (stored as 0)
+        fr[7, 11, 22] = np.nan
     (a, na), (b, _) = lists(st, fr, t, f, (RUNS[storage], 1), normalize=normalize,
                             storage=storage)
     assert ("runs" in na) == (scale == 1.0)
     same(a, b)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("W", [96, 93])
+def test_raw_nan_pixels_reach_only_their_own_stacks(st, storage, W):
+    # a NaN beside the mover's path, in an early and in a late frame: the
+    # stacks that never read it keep their values
+    for i in (0, 19, 39):
+        fr, t, f = field(6, W=W, nvx=24, nvy=20, N=40)
+        p = [f[k] for k in ("vx0", "dvx", "vy0", "dvy", "t_ref")]
+        x = round(W * 0.4 + 3 * p[1] * (t[i] - p[4]))
+        y = round(f["height"] * 0.5 - 2 * p[3] * (t[i] - p[4]))
+        fr[i, y + 1, x] = fr[i, y - 1, x] = fr[i, y, x + 2] = np.nan
+        (a, na), (b, _) = lists(st, fr, t, f, (RUNS[storage], 1), normalize=False, storage=storage)
+        assert "runs" not in na
+        same(a, b)
 
 
 def test_runs_infinite_pixels(st):
