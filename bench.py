@@ -45,21 +45,23 @@ METRIC = "G pixel*frame*velocity adds/s (2048x2048x256, 801x801 grid)"
 
 # DRAM bytes (read + write) of one stack-kernel launch, from one ncu capture
 # of `--metrics dram__bytes_read.sum,dram__bytes_write.sum` (profiles/
-# stack_speculoos_2048x256_traffic.md), keyed by workload, storage, sampling
-# and the kernel variant that ran, with the SHA-1 prefix of the kernel's code
-# it was taken on (k_stack_fast.cu and its generated PTX bodies, comments and
-# blank lines removed, so only a change of the code itself retires the
-# figure): reported only while the code is that one.
+# stack_runs_1024x64_ncu.md), keyed by workload, storage, sampling and the
+# kernel variant that ran, with the SHA-1 prefix of the kernel's code it was
+# taken on (its source and generated PTX bodies, comments and blank lines
+# removed, so only a change of the code itself retires the figure): reported
+# only while the code is that one.
 STACK_TRAFFIC = {
-    ("speculoos", "f32", "nearest", "float_ky8_s2_f16_cpfalse_o48_h1"):
-        (45.867799296e9 + 370.29248e6, "119452094ca3"),
+    ("speculoos", "f32", "nearest", "float_runs_ky8_x4_s3_f16"):
+        (263.554441728e9 + 26.86097664e9, "236fdd105713"),
 }
 
 
-def stack_source_sha():
+def stack_source_sha(variant):
     import hashlib
     code = []
-    for name in ("k_stack_fast.cu", "st_bodies.inc"):
+    names = ("k_stack_runs.cu", "st_runs.inc") if "_runs_" in variant \
+        else ("k_stack_fast.cu", "st_bodies.inc")
+    for name in names:
         path = os.path.join(ROOT, "paper_2303_07293_gb300", "csrc", name)
         with open(path) as fh:
             for line in fh:
@@ -744,17 +746,17 @@ def main():
     variant = plan.stack_variant_name(0)
     config["stack_variant"] = variant
     tr = STACK_TRAFFIC.get((args.workload, args.storage, args.mode, variant))
-    traffic = tr[0] if tr and tr[1] == stack_source_sha() and stack_launch == args.steps \
+    traffic = tr[0] if tr and tr[1] == stack_source_sha(variant) and stack_launch == args.steps \
         and (args.width, args.frames, args.nv) == (None, None, None) else None
     if traffic is not None:
         traffic_note = "DRAM bytes of one launch from the stored ncu capture of this code"
     elif tr is None:
         traffic_note = (f"null: no ncu DRAM capture stored for this workload and variant "
                         f"({variant})")
-    elif tr[1] != stack_source_sha():
+    elif tr[1] != stack_source_sha(variant):
         traffic_note = (f"null: the stored capture ({tr[0] / 1e9:.2f} GB per launch) was taken "
-                        f"on k_stack_fast.cu code {tr[1]}, the kernel is now "
-                        f"{stack_source_sha()}")
+                        f"on kernel code {tr[1]}, the kernel is now "
+                        f"{stack_source_sha(variant)}")
     else:
         traffic_note = "null: the stored capture is of one launch per step"
     # algorithmic work per pixel*frame*velocity: 1 add (nearest), 4 FMA (bilinear)
@@ -764,6 +766,9 @@ def main():
             "unit": "T FMA/s" if args.mode == "bilinear" else "T adds/s",
             "frac": achieved / peak_t, "traffic": traffic, "traffic_note": traffic_note,
             "work_per_unit": per_unit,
+            "work_note": "adds of the plain definition, N per pixel and velocity; the runs "
+                         "variant sums frames with equal relative shifts once and makes "
+                         "fewer than a third of them, so frac can exceed 1",
             "kernel": "stack (shift-and-stack + threshold)", "launches_per_step":
                 stack_launch / args.steps, "avg_launch_ms": stack_avg_ms,
             "peak_basis": f"{sms} SMs x 128 FP32 lanes x {max_mhz:.0f} MHz (max SM clock)"}
