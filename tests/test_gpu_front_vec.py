@@ -40,3 +40,25 @@ def test_sums_and_bins_bitexact(st, N, H, W, lead):
     out = st.bin2x2(x)
     assert tuple(out.shape) == ref.shape
     assert np.array_equal(out.cpu().numpy(), ref, equal_nan=True)
+
+
+@pytest.mark.parametrize("lead", [0, 1, 4])
+@pytest.mark.parametrize("N,H,W", [(1, 1, 4), (2, 3, 44), (3, 7, 9), (5, 1, 127), (8, 2, 66),
+                                   (33, 4, 33), (50, 3, 172), (63, 5, 51), (64, 2, 130),
+                                   (65, 2, 66), (97, 1, 40), (200, 3, 31), (600, 1, 68)])
+def test_medians_bitexact(st, N, H, W, lead):
+    # masked and infinite samples, whole columns of them, zeros of both signs
+    rng = np.random.default_rng(100 * N + W)
+    fr = rng.standard_normal((N, H, W)).astype(np.float32)
+    hide = rng.random(fr.shape) < rng.random((H, W)) - 0.4
+    fr[hide] = rng.choice(np.array([np.nan, np.inf, -np.inf], np.float32), int(hide.sum()))
+    fr[:, 0, 0], fr[:, 0, 1] = np.nan, np.float32(-0.0)
+    fr[N // 2:, H - 1, W - 1] = 0.0
+    buf = torch.zeros(lead + fr.size, device="cuda")
+    x = buf[lead:].view(N, H, W)
+    x.copy_(torch.from_numpy(fr))
+    with np.errstate(invalid="ignore"):
+        ref, rmed = front.median_subtract(fr)
+    out, med = st.median_subtract(x, with_median=True)
+    assert np.array_equal(med.cpu().numpy(), rmed, equal_nan=True)
+    assert np.array_equal(out.cpu().numpy(), ref, equal_nan=True)
