@@ -36,9 +36,11 @@ namespace {
 // spacing at the median: 10 steps for noise) or the bracket is one value.  No
 // step moves data or branches on it.  Masked samples are the highest key and
 // never counted.
+// Frames that all start on 16 bytes are moved 16 bytes a lane, in and out, as
+// 4-byte pieces kept too few bytes in flight.
 // What bounds it: the counting, about 12 steps x N x 2 instructions a pixel,
-// against 8 N bytes.  1024^2 x 200: 0.645 ms, 2.6 TB/s (quickselect in
-// shared memory, one warp a block: 6.5 ms).
+// against 8 N bytes.  1024^2 x 200: 0.498 ms, 3.4 TB/s (4-byte pieces 0.645;
+// quickselect in shared memory, one warp a block: 6.5 ms).
 constexpr int kMedPix = 32, kMedShare = 8, kMedPitch = 36;
 
 __device__ __forceinline__ int32_t med_key(float x) {
@@ -65,13 +67,25 @@ __device__ __forceinline__ int max8(int v) { return ~min8(~v); }
 // has its pixels' whole columns in shared memory before it writes any of them.
 template <int K>
 __global__ void __launch_bounds__(kMedPix * kMedShare)
-    k_median_long(const float* in, int N, int64_t P, float* out, float* __restrict__ median) {
-  extern __shared__ float sm[];  // [N][kMedPitch] samples in frame order, [32] medians
+    k_median_long(const float* in, int N, int64_t P, float* out, float* __restrict__ median,
+                  const bool vec) {
+  extern __shared__ __align__(16) float sm[];  // [N][kMedPitch] samples in frame order, [32] medians
   float* med_sh = sm + (size_t)N * kMedPitch;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t p0 = (int64_t)blockIdx.x * kMedPix;
-  {
-    const bool ok = p0 + lane < P;  // (a pixel past the end reads zeros)
+  // (a pixel past the end reads zeros)
+  const int row4 = tid / 8, off4 = tid % 8 * 4;  // 16-byte pieces: 8 lanes a frame
+  const bool ok4 = p0 + off4 < P;
+  if (vec) {
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sm + off4);
+    const float* src = ok4 ? in + p0 + off4 : in;
+    for (int i = row4; i < N; i += kMedPix)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                       dst + (uint32_t)(i * kMedPitch * 4)),
+                   "l"(src + (int64_t)i * P), "r"(ok4 ? 16 : 0)
+                   : "memory");
+  } else {
+    const bool ok = p0 + lane < P;
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sm + lane);
     for (int i = warp; i < N; i += kMedShare) {
       const float* src = ok ? in + (int64_t)i * P + p0 + lane : in;
@@ -80,9 +94,9 @@ __global__ void __launch_bounds__(kMedPix * kMedShare)
                    "l"(src), "r"(ok ? 4 : 0)
                    : "memory");
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   // lane = 8 pixel + share, 4 pixels a warp
   const int px = 4 * warp + (lane >> 3), share = lane & 7;
@@ -149,9 +163,20 @@ __global__ void __launch_bounds__(kMedPix * kMedShare)
   if (share == 0) med_sh[px] = med;
   __syncthreads();
   const int64_t p = p0 + lane;
+  if (median && warp == 0 && p < P) median[p] = med_sh[lane];
+  if (vec) {
+    if (!ok4) return;
+    const float4 m = *reinterpret_cast<const float4*>(med_sh + off4);
+    for (int i = row4; i < N; i += kMedPix) {
+      const float4 v = *reinterpret_cast<const float4*>(sm + i * kMedPitch + off4);
+      __stcs(reinterpret_cast<float4*>(out + (int64_t)i * P + p0 + off4),
+             make_float4(__fsub_rn(v.x, m.x), __fsub_rn(v.y, m.y), __fsub_rn(v.z, m.z),
+                         __fsub_rn(v.w, m.w)));
+    }
+    return;
+  }
   if (p >= P) return;
   med = med_sh[lane];
-  if (median && warp == 0) median[p] = med;
   for (int i = warp; i < N; i += kMedShare)
     out[(int64_t)i * P + p] = __fsub_rn(sm[i * kMedPitch + lane], med);
 }
@@ -246,11 +271,13 @@ int launch_median_subtract(const float* in, int N, int64_t P, float* out, float*
   const int64_t blocks = (P + kMedPix - 1) / kMedPix;
   if (blocks > 0x7fffffff) return -1;
   const size_t smem = ((size_t)N * kMedPitch + kMedPix) * sizeof(float);
+  const bool vec = P % 4 == 0 && on_16(in) && on_16(out);
 #define ST_MED(K)                                                                              \
   if (N <= kMedShare * K) {                                                                    \
     cudaFuncSetAttribute((const void*)k_median_long<K>,                                        \
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);              \
-    k_median_long<K><<<(unsigned)blocks, kMedPix * kMedShare, smem, s>>>(in, N, P, out, median); \
+    k_median_long<K><<<(unsigned)blocks, kMedPix * kMedShare, smem, s>>>(in, N, P, out, median, \
+                                                                         vec);                 \
     return 1;                                                                                  \
   }
   ST_MED(12) ST_MED(16) ST_MED(20) ST_MED(24) ST_MED(28) ST_MED(32) ST_MED(40) ST_MED(48) ST_MED(64)
