@@ -56,7 +56,7 @@ STACK_TRAFFIC = {
 }
 
 
-def stack_source_sha(variant):
+def stack_source_sha(variant="_runs_"):
     import hashlib
     code = []
     names = ("k_stack_runs.cu", "st_runs.inc") if "_runs_" in variant \
