@@ -30,20 +30,23 @@
 // owns cutout column t%64 and its 16 rows (t/64)*16.., so a warp reads 32
 // consecutive words of a box row, and handles its rows in pairs (k, k + 8):
 // tap rows q and q + 8 are one register pair, so the differences d = a1 - a0,
-// the horizontal interpolations h = a0 + fx d, their steps e = h' - h and the
-// sums are paired FP32 operations; the slope along x, whose weights (1 - fy)
-// and fy are the frame's, is summed as <g, d> and <g, d'>.  A ninth warp forms a
+// the horizontal interpolations h = a0 + fx d, their steps e = h' - h, the
+// slopes and the sums S are paired FP32 operations; a frame's <g, slope> is
+// added up row by row (a change of its rounding alone moves a Gauss-Newton
+// path across the kinks of the bilinear stack).  A ninth warp forms a
 // frame's shift when it issues the copy and leaves the fractions beside it;
 // each consumer warp releases a slot by itself (a consumer that issues the
-// copies paces all others: 48 ms).  Reductions use a fixed-order block tree.  Every wait is
+// copies paces all others: 51 ms against 48).  Reductions use a fixed-order block tree.  Every wait is
 // bounded in time.
 //
-// What bounds it: per frame and cutout 272 shared-memory wavefronts and 66
-// paired operations a warp on the FP32 pipe, which paired FMAs of three distinct
-// register pairs reach at 0.67 of its rate (measured: 85 against 127 for adds, in
-// operations per clock and SM): about 400 clocks of the 590 it takes.  Half the
+// What bounds it: per frame and cutout 272 shared-memory wavefronts and 58
+// paired and 32 single operations a warp on the FP32 pipe, which paired FMAs of
+// three distinct register pairs reach at 0.67 of its rate (measured: 85 against
+// 127 for adds, in operations per clock and SM): about 400 clocks of the 600 it
+// takes.  Half the
 // rows copied, 3 or 5 stages or three CTAs an SM: the same time.  4096
-// candidates x 300 frames x 21 evaluations: 62.5 ms with scalar operations, 48.2.
+// candidates x 300 frames x 21 evaluations: 62.5 ms with scalar operations, 50.1 (48.2 with
+// the slopes' sums paired too).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -392,7 +395,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_refine(RefineArgs a) {
       const float2 neg = make_float2(-1.0f, -1.0f);
       // tap rows q and q + 8 of the column and its right neighbour
       float2 hp, dp;
-      float2 ga = make_float2(0.0f, 0.0f), gb = ga, ge = ga;  // <g, d>, <g, d'>, <g, e>
+      // <g, slope in x> and <g, slope in y> in row order: rows 0..7 as they come,
+      // then rows 8..15, whose slopes wait in registers
+      float gdx = 0.0f, gdy = 0.0f, sx[kHalf], sy[kHalf];
 #pragma unroll
       for (int k = 0; k <= kHalf; ++k) {
         const T* r = box + k * kBoxW;
@@ -404,18 +409,24 @@ __global__ void __launch_bounds__(kBlock, 2) k_refine(RefineArgs a) {
         if (k > 0) {
           const float2 e = __ffma2_rn(hp, neg, h);
           S2[k - 1] = __fadd2_rn(S2[k - 1], __ffma2_rn(fy2, e, hp));
-          ga = __ffma2_rn(g2[k - 1], dp, ga);
-          gb = __ffma2_rn(g2[k - 1], d, gb);
-          ge = __ffma2_rn(g2[k - 1], e, ge);
+          const float2 u = __ffma2_rn(fy2, __ffma2_rn(dp, neg, d), dp);  // (1-fy) dp + fy d
+          gdx = __fmaf_rn(g2[k - 1].x, u.x, gdx);
+          gdy = __fmaf_rn(g2[k - 1].x, e.x, gdy);
+          sx[k - 1] = u.y;
+          sy[k - 1] = e.y;
         }
         hp = h;
         dp = d;
       }
       __syncwarp();
       if ((tid & 31) == 0) mbar_arrive(&empty[slot]);
-      const float va = ga.x + ga.y, vb = gb.x + gb.y;
-      dvx += fr.z * (va + fr.y * (vb - va));
-      dvy += fr.z * (ge.x + ge.y);
+#pragma unroll
+      for (int k = 0; k < kHalf; ++k) {
+        gdx = __fmaf_rn(g2[k].y, sx[k], gdx);
+        gdy = __fmaf_rn(g2[k].y, sy[k], gdy);
+      }
+      dvx += fr.z * gdx;
+      dvy += fr.z * gdy;
     }
     ok = __syncthreads_and(ok);
     if (!ok) {
