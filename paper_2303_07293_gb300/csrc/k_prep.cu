@@ -377,7 +377,8 @@ __global__ void __launch_bounds__(kSkyThreads, 4)
                SkyPartial* __restrict__ partial) {
   __shared__ SkyPartial sh[kSkyThreads / 32];
   __shared__ SkyState s_st;
-  __shared__ bool s_flag;
+  // (two flags: a warp that still has to read the first must not see the second)
+  __shared__ bool s_last, s_again;
   const int i = blockIdx.y, tid = threadIdx.x;
   SkyState st = state[i];
   if (st.done) return;  // frame converged (uniform per block)
@@ -394,10 +395,10 @@ __global__ void __launch_bounds__(kSkyThreads, 4)
   if (tid == 0) {
     mine[blockIdx.x] = a;
     __threadfence();
-    s_flag = atomicAdd(&state[i].arrived, 1u) == blocks - 1;
+    s_last = atomicAdd(&state[i].arrived, 1u) == blocks - 1;
   }
   __syncthreads();
-  if (!s_flag) return;
+  if (!s_last) return;
   __threadfence();
   if (tid < 32) {
     auto load = [&](int b) {
@@ -418,17 +419,17 @@ __global__ void __launch_bounds__(kSkyThreads, 4)
   // by this block: rare, and the next membership depends on it
   for (int again = 0;; ++again) {
     if (tid == 0) {
-      s_flag = false;
+      s_again = false;
       if (a.n > 0) {
         sky_moments(a, st);
         SkyState nx = st;
         set_range(nx, nx.mu, (kKappa + 0.1) * nx.sigma);
-        s_flag = again < 4 && ldexp(1.0, st.r) > 64.0 * st.sigma && nx.r < st.r;
+        s_again = again < 4 && ldexp(1.0, st.r) > 64.0 * st.sigma && nx.r < st.r;
         s_st = nx;
       }
     }
     __syncthreads();
-    if (!s_flag) break;
+    if (!s_again) break;
     st = s_st;
     a = sky_sums(f, 0, nvec, st, sh);
     __syncthreads();
