@@ -70,7 +70,7 @@ struct FieldPlan {
   float* d_rsq = nullptr;
   void* d_cube = nullptr;        // normalised / converted storage cube (owned)
   int pitch = 0;                 // its row pitch: a multiple of 16 bytes
-  bool copied = false;           // it is a plain copy of the frames with that pitch
+  bool copies = false;           // d_cube, if any, is a plain copy of the frames with that pitch
   float* d_frames_copy = nullptr; // device copy for the host-buffer entry point
   FastPlan* fast = nullptr;
   int last_variant = -1;
@@ -326,6 +326,22 @@ FieldDev field_dev(const FieldPlan& fp, const float* d_frames, int fi, int stora
   return d;
 }
 
+// Takes or gives back the padded copy of frames that are used as given: held
+// while the motion fits the kernels that read it, and taken only if it leaves
+// the caller at least as much device memory as it takes.
+void hold_copy(FieldPlan& fp, bool wanted) {
+  const size_t bytes = sizeof(float) * (size_t)fp.f.n_frames * fp.pitch * (size_t)fp.f.height;
+  size_t avail = 0, total = 0;
+  if (!wanted) {
+    cudaFree(fp.d_cube);
+    fp.d_cube = nullptr;
+  } else if (!fp.d_cube && cudaMemGetInfo(&avail, &total) == cudaSuccess && bytes <= avail / 2 &&
+             cudaMalloc(&fp.d_cube, bytes) != cudaSuccess) {
+    fp.d_cube = nullptr;
+    cudaGetLastError();
+  }
+}
+
 // plain: with the default kernel that passes on the fewest points (the pending
 // list overflowed).
 st_status device_search(st_plan_t* p, const float* const* d_frames, const double* const* h_times,
@@ -361,12 +377,13 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
       CK(cudaGetLastError());
       fp.fast_fits = fits;
       fp.fast_ready = true;
+      if (fp.copies) {
+        hold_copy(fp, fits);
+        fds[fi] = field_dev(fp, d_frames[fi], fi, p->o.storage);
+      }
     }
-    use_fast[fi] = fp.fast && fp.fast_fits;
-    if (fp.copied && !use_fast[fi]) {  // the direct gather reads the frames as they are
-      fds[fi].cube = d_frames[fi];
-      fds[fi].pitch = fp.f.width;
-    }
+    // (without a copy the direct gather reads the frames as they are)
+    use_fast[fi] = fp.fast && fp.fast_fits && !(fp.copies && !fp.d_cube);
     if (use_fast[fi]) {
       fast_fds.push_back(fds[fi]);
       fast_fps.push_back(fp.fast);
@@ -691,21 +708,18 @@ st_status st_plan(const st_field* fields, int32_t n_fields, const st_opts* opts,
     // kernels 4)
     const int align = opts->storage == ST_F32 ? 4 : 8;
     fp.pitch = (f.width + align - 1) / align * align;
-    const size_t cube_bytes =
-        store_bytes(opts->storage) * (size_t)f.n_frames * fp.pitch * (size_t)f.height;
-    if (opts->normalize || opts->storage != ST_F32) {
-      guard(cudaMalloc(&fp.d_cube, cube_bytes), "cudaMalloc(cube)");
-    } else if (fp.pitch != f.width && opts->tile != 1 && fp.nk() >= 128 && f.n_frames >= 8) {
-      // frames used as given, of another width: a padded copy, if it fits the
-      // memory and the grid repays it (a pass takes as long as about 40
+    if (opts->normalize || opts->storage != ST_F32)
+      guard(cudaMalloc(&fp.d_cube, store_bytes(opts->storage) * (size_t)f.n_frames * fp.pitch *
+                                       (size_t)f.height),
+            "cudaMalloc(cube)");
+    else
+      // frames used as given, of another width: a padded copy, made where the
+      // motion fits and the grid repays it (a pass takes as long as about 40
       // velocities' stacks)
-      if (cudaMalloc(&fp.d_cube, cube_bytes) == cudaSuccess)
-        fp.copied = true;
-      else
-        cudaGetLastError();
-    }
+      fp.copies = fp.pitch != f.width && opts->tile != 1 && fp.nk() >= 128 && f.n_frames >= 8;
     if (st == ST_OK && opts->tile != 1) {
       FieldDev probe = field_dev(fp, nullptr, i, opts->storage);
+      if (fp.copies) probe.pitch = fp.pitch;
       if (fast_eligible(probe, opts->mode) && !fast_plan_build(probe, opts->mode, &fp.fast))
         st = fail(ST_ERR_OOM, "field %d: fast-kernel tables could not be allocated", i);
       if (fp.fast && opts->tile >= 2) fast_set_variant(fp.fast, opts->tile - 2);
@@ -869,7 +883,9 @@ st_status st_dump_stack(st_plan_t* p, int32_t field, const float* d_frames, cons
   for (int q = 0; q < n_k && whole; ++q) whole = h_k[q] == q;
   if (e == cudaSuccess) {
     int n = -1;
-    if (whole && fp.fast) {
+    // (its tensor map needs rows of whole 16 bytes: not the frames of a padded
+    // copy that is not held)
+    if (whole && fp.fast && fast_eligible(fd, p->o.mode)) {
       bool fits = false;
       fast_prepare(fd, fp.fast, p->s, &fits);
       if (fits)

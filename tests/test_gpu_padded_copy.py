@@ -32,7 +32,7 @@ def test_copy_is_held_only_while_it_is_read(st, mode):
     copy = 4 * N * H * (W + 1)
     slow = np.linspace(0.0, 2.0, N)
     fast = slow * 40.0   # adjacent velocities many pixels apart
-    f = synth.field_params(W, H, N, 0.0, -0.4 * (nv // 2), 0.4, nv, -0.4 * (nv // 2), 0.4, nv,
+    f = synth.field_params(W, H, N, 0.0, -0.2 * (nv // 2), 0.2, nv, -0.2 * (nv // 2), 0.2, nv,
                            tau=5.0)
     got = {}
     for tile in (1, 0):
@@ -51,3 +51,26 @@ def test_copy_is_held_only_while_it_is_read(st, mode):
             assert p.last_stack_variant(0) == 0
     for a, b in zip(got[0], got[1]):
         assert a.tobytes() == b.tobytes()
+
+
+def test_copy_leaves_as_much_memory_as_it_takes(st):
+    # less than twice the copy is free: the direct gather reads the frames
+    N, H, W, nv = 40, 1021, 1023, 13
+    x = torch.randn((N, H, W), device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    copy = 4 * N * H * (W + 1)
+    t = np.linspace(0.0, 2.0, N)
+    f = synth.field_params(W, H, N, 0.0, -0.2 * (nv // 2), 0.2, nv, -0.2 * (nv // 2), 0.2, nv,
+                           tau=5.0)
+    with st.Plan(f) as p:
+        want = p.candidates(x, t)
+        assert p.last_stack_variant(0) == 1
+    with st.Plan(f, tile=1) as p:
+        p.candidates(x, t)
+    torch.cuda.empty_cache()
+    with st.Plan(f) as p:
+        hold = torch.empty(int(free() - 1.6 * copy), dtype=torch.uint8, device="cuda")
+        got = p.candidates(x, t)
+        assert p.last_stack_variant(0) == 0
+        del hold
+        torch.cuda.empty_cache()
+    assert got.tobytes() == want.tobytes()
