@@ -1329,10 +1329,8 @@ bool fast_plan_build(const FieldDev& fd, int mode, FastPlan** out) {
               cudaMalloc(&fp->d_pat, (size_t)fd.N * fp->nB) == cudaSuccess &&
               cudaMalloc(&fp->d_ff, sizeof(FastField)) == cudaSuccess &&
               cudaMalloc(&fp->d_map, sizeof(CUtensorMap)) == cudaSuccess;
-  if (good && vr >= 0) {
-    fp->run = run_plan_build(fd, fp->nB);
-    good = fp->run != nullptr;
-  }
+  // (without the run kernel's tables another variant does its work)
+  if (good && vr >= 0 && !(fp->run = run_plan_build(fd, fp->nB))) cudaGetLastError();
   if (!good) {
     fast_plan_free(fp);
     return false;
