@@ -179,7 +179,8 @@ void st_free(st_plan_t* plan);
  * buffer succeeds.  Returns ST_ERR_OVERFLOW with *h_count = -1 when the
  * above-threshold points exceed the plan's pending_capacity (the default
  * variant's filter is wider than the threshold by its rounding margin: if its
- * points do not fit, the search is run again with a frame-order variant), and
+ * points do not fit, the search is run again with a frame-order variant, which
+ * searches at the same timestamps then start with), and
  * ST_ERR_TIMEOUT (*h_count = -1) when a pipeline wait of the stack kernel
  * gave up after 2 s (the device stays usable).  Every field whose motion fits
  * the register-window kernel is searched in one persistent launch; shift

@@ -1576,6 +1576,10 @@ bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, bool plain, cu
          nullptr;
 }
 
+bool fast_plain_differs(const FieldDev* fds, FastPlan* const* fps, int n, bool runs) {
+  return runs || plain_variant(fds, fps, n, true) != plain_variant(fds, fps, n, false);
+}
+
 void fast_note_ran(const FieldDev* fds, FastPlan* const* fps, int n, bool runs) {
   const int vi = runs ? fps[0]->variant : plain_variant(fds, fps, n, true);
   for (int i = 0; i < n; ++i) fps[i]->ran = vi;

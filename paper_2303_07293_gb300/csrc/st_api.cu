@@ -128,6 +128,7 @@ struct st_plan_s {
   uint64_t gen = 1;             // bumped when tables, variants or maps change
   int64_t graph_stack_launches = 0;
   int64_t graph_launches = 0;
+  bool plain = false;             // the margin's points do not fit the pending list
   bool graph_broken = false;    // capture failed once: run directly
   bool last_replayed = false;
 };
@@ -342,11 +343,17 @@ void hold_copy(FieldPlan& fp, bool wanted) {
   }
 }
 
-// plain: with the default kernel that passes on the fewest points (the pending
-// list overflowed).
+// What a search's first pass took, where a second follows.
+struct Redo {
+  double stack_ms;
+  int64_t stack_launches, launches;
+};
+
+// redo: the second pass, with the default kernel that passes on the fewest
+// points (the pending list overflowed).
 st_status device_search(st_plan_t* p, const float* const* d_frames, const double* const* h_times,
                         st_candidate* d_out, int64_t capacity, int64_t* h_count,
-                        bool plain = false) {
+                        const Redo* redo = nullptr) {
   if (!d_frames || !h_times || !h_count) return fail(ST_ERR_INVALID, "NULL argument");
   if (capacity < 0 || (capacity > 0 && !d_out))
     return fail(ST_ERR_INVALID, "capacity must be >= 0 and d_out non-NULL when capacity > 0");
@@ -355,14 +362,16 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     if (!d_frames[fi]) return fail(ST_ERR_INVALID, "field %d: frames are NULL", fi);
   // ---- host-side preparation: tables (when the timestamps change), the
   // register-window tables and variant, the tensor maps
-  int64_t L = 0;
+  int64_t L = redo ? redo->launches : 0;
   std::vector<FieldDev> fds(nf);
   for (int fi = 0; fi < nf; ++fi) {
     bool changed = false;
     st_status st = prepare_tables(p, fi, h_times[fi], &L, &changed);
     if (st != ST_OK) return st;
+    if (changed) p->plain = false;
     fds[fi] = field_dev(p->F[fi], d_frames[fi], fi, p->o.storage);
   }
+  const bool plain = redo || p->plain;
   // fields that fit the register-window kernel run in one persistent launch;
   // its variant is tuned (or looked up) on the field with the most work
   std::vector<char> use_fast(nf, 0);
@@ -509,7 +518,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   int64_t stack_launches = 0, dev_launches = 0;
   p->last_replayed = false;
   bool done = false;
-  if (p->o.use_graph && !p->graph_broken && !plain) {
+  if (p->o.use_graph && !p->graph_broken && !redo) {
     std::vector<const float*> key(d_frames, d_frames + nf);
     if (!(p->graph && p->graph_gen == p->gen && p->graph_frames == key)) {
       // capture the device part once for these frames and tables
@@ -570,13 +579,21 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   CK(cudaStreamSynchronize(p->s));
   float ms = 0.0f;
   CK(cudaEventElapsedTime(&ms, p->e0, p->e1));
-  p->stack_ms = ms;
-  p->stack_launches = stack_launches;
+  p->stack_ms = ms + (redo ? redo->stack_ms : 0.0);
+  p->stack_launches = stack_launches + (redo ? redo->stack_launches : 0);
   Counters c = *p->h_ctr;
   if (runs)
     fast_note_ran(fast_fds.data(), fast_fps.data(), (int)fast_fps.size(), c.runs != 0);
-  if ((c.error & ERR_PENDING_OVERFLOW) && !plain && !fast_fds.empty())
-    return device_search(p, d_frames, h_times, d_out, capacity, h_count, true);
+  if ((c.error & ERR_PENDING_OVERFLOW) && !plain && !fast_fds.empty() &&
+      fast_plain_differs(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(), c.runs != 0)) {
+    const Redo first{p->stack_ms, p->stack_launches, L};
+    return device_search(p, d_frames, h_times, d_out, capacity, h_count, &first);
+  }
+  if (redo && !(c.error & ERR_PENDING_OVERFLOW)) {
+    // the points fit but for the margin's: searches at these times start here
+    p->plain = true;
+    ++p->gen;  // (a captured graph runs the first pass)
+  }
   if (c.error & ERR_PENDING_OVERFLOW) {
     *h_count = -1;
     p->launches = L;

@@ -145,6 +145,9 @@ struct RunCtl {
   const int* d_use;
 };
 bool fast_runs_chosen(const FieldDev* fds, FastPlan* const* fps, int n);
+// Whether a launch without a RunCtl runs another variant than one with it did
+// (runs: the run kernel).
+bool fast_plain_differs(const FieldDev* fds, FastPlan* const* fps, int n, bool runs);
 // Notes which of the two a launch with d_use ran (for the variant's name).
 void fast_note_ran(const FieldDev* fds, FastPlan* const* fps, int n, bool runs);
 int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, float* dump_S,

@@ -60,11 +60,10 @@ def test_margin_that_does_not_fit_is_found_out_once(st, graph):
         assert passes == [2, 1, 1, 1]   # both passes counted; then the one that fits
         assert p.last_graph_replayed() == graph
         # other times: the margin is tried again
-        t2 = t * 0.97
-        got = p.candidates(x, t2)
-        assert p.last_stack_kernel_time()[1] in (1, 2)
-        with st.Plan(f, tile=2, **kw) as q:
-            assert got.tobytes() == q.candidates(x, t2).tobytes()
+        t2 = t + 1e-12
+        for expect in (2, 1):
+            assert p.candidates(x, t2).tobytes() == want.tobytes()
+            assert p.last_stack_kernel_time()[1] == expect
     with st.Plan(f, tile=9, use_graph=graph, **kw) as p:   # room for the margin: one pass
         p.candidates(x, t)
         assert p.last_stack_kernel_time()[1] == 1 and "runs" in p.stack_variant_name(0)
@@ -73,9 +72,9 @@ def test_margin_that_does_not_fit_is_found_out_once(st, graph):
 @pytest.mark.parametrize("mode,tile", [("nearest", 2), ("nearest", 4), ("nearest", 1),
                                        ("bilinear", 0)])
 def test_overflow_is_reported_after_one_pass(st, mode, tile):
-    # far more points than the list holds: the search takes no longer than one
-    # that succeeds (half as long again for the clock's sake)
-    x, t, f = field(W=512, H=512, N=48, nv=32, tau=3.0)
+    # a few more points than the list holds: the search takes no longer than
+    # one that succeeds (half as long again for the clock's sake)
+    x, t, f = field(W=512, H=512, N=48, nv=64, tau=4.7)
     kw = dict(mode=mode, tile=tile, normalize=True, cr_clip=10.0)
     best = {}
     for cap in (1, 1 << 22):
