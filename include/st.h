@@ -180,7 +180,11 @@ void st_free(st_plan_t* plan);
  * above-threshold points exceed the plan's pending_capacity (the default
  * variant's filter is wider than the threshold by its rounding margin: if its
  * points do not fit, the search is run again with a frame-order variant, which
- * searches at the same timestamps then start with), and
+ * searches at the same timestamps then start with; with bilinear sampling the
+ * register-window kernel's filter is wider by a bound of its rounding for the
+ * field's largest value, and a field that holds an infinity, one whose bound
+ * would be too wide, or one whose points do not fit for it, is searched again
+ * by the direct-gather kernel), and
  * ST_ERR_TIMEOUT (*h_count = -1) when a pipeline wait of the stack kernel
  * gave up after 2 s (the device stays usable).  Every field whose motion fits
  * the register-window kernel is searched in one persistent launch; shift

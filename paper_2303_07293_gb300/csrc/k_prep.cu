@@ -539,9 +539,14 @@ __device__ __forceinline__ float normalize_pair(float r, const NormFrame& f, boo
 }
 
 // |v|'s bits, which order as the magnitudes do, an infinity above the finite
-// ones and a NaN above both: the run kernel's moves between running sums carry
-// either to outputs that never read the pixel, so both have to reach the margin.
-__device__ __forceinline__ unsigned mag(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+// ones and a NaN above both.  The run kernel's moves between running sums carry
+// either to outputs that never read the pixel, so both have to reach its
+// margin; in the other kernels a NaN stays with the outputs that read it, as in
+// the direct gather, and counts as 0.
+__device__ __forceinline__ unsigned mag(float v, bool nan) {
+  const unsigned b = __float_as_uint(v) & 0x7fffffffu;
+  return b > 0x7f800000u && !nan ? 0u : b;
+}
 
 // The warps' largest magnitude into *absmax.
 __device__ __forceinline__ void put_max(unsigned top, unsigned* absmax) {
@@ -550,35 +555,37 @@ __device__ __forceinline__ void put_max(unsigned top, unsigned* absmax) {
 }
 
 __global__ void __launch_bounds__(256)
-    k_absmax(const float* __restrict__ x, int64_t n, unsigned* __restrict__ absmax) {
+    k_absmax(const float* __restrict__ x, int64_t n, bool nan, unsigned* __restrict__ absmax) {
   const int64_t head = min(n, (int64_t)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15) / 4);
   const float4* v = reinterpret_cast<const float4*>(x + head);
   const int64_t nv = (n - head) / 4, tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned top = 0u;
-  if (tid < head) top = mag(x[tid]);
-  if (tid < n - head - 4 * nv) top = max(top, mag(x[head + 4 * nv + tid]));
+  if (tid < head) top = mag(x[tid], nan);
+  if (tid < n - head - 4 * nv) top = max(top, mag(x[head + 4 * nv + tid], nan));
 #pragma unroll 4
   for (int64_t j = tid; j < nv; j += (int64_t)gridDim.x * blockDim.x) {
     const float4 q = __ldg(v + j);
-    top = max(top, max(max(mag(q.x), mag(q.y)), max(mag(q.z), mag(q.w))));
+    top = max(top, max(max(mag(q.x, nan), mag(q.y, nan)), max(mag(q.z, nan), mag(q.w, nan))));
   }
   put_max(top, absmax);
 }
 
-__global__ void k_run_margins(const FieldDev* __restrict__ fds, int n,
-                              const unsigned* __restrict__ absmax, float* __restrict__ margin,
-                              int* __restrict__ use) {
+__global__ void k_margins(const FieldDev* __restrict__ fds, int n, int mode,
+                          const unsigned* __restrict__ absmax, float* __restrict__ margin,
+                          int* __restrict__ use, Counters* __restrict__ ctr) {
   const int f = threadIdx.x;
   bool ok = true;
   if (f < n) {
     const FieldDev& d = fds[f];
-    // (a 16-bit value may be larger than the value it was rounded from)
-    const float m = run_margin(1.01f * __uint_as_float(absmax[f]), d.N, d.thr[d.N]);
+    const float m = margin_of(mode, __uint_as_float(absmax[f]), d.N, d.thr[d.N]);
     margin[f] = m;
-    ok = run_margin_ok(m, d.nmin, d.thr[d.nmin]);
+    ok = margin_ok(mode, m, d.nmin, d.thr[d.nmin]);
   }
   const int all = __syncthreads_and(ok);
-  if (f == 0) *use = all;
+  if (f == 0) {
+    *use = all;
+    if (!all && mode == ST_BILINEAR) atomicOr(&ctr->error, ERR_MARGIN);
+  }
 }
 
 template <typename T>
@@ -586,7 +593,7 @@ __global__ void __launch_bounds__(256)
     k_normalize_store(const float* __restrict__ raw, int W, int H, int normalize, float cr_clip,
                       const SkyState* __restrict__ state, T* __restrict__ cube, int pitch,
                       double* __restrict__ mu_out, double* __restrict__ sigma_out,
-                      unsigned* __restrict__ absmax) {
+                      unsigned* __restrict__ absmax, bool nan) {
   const int i = blockIdx.y;
   const int64_t npix = (int64_t)W * H;
   const float* x = raw + (int64_t)i * npix;
@@ -644,10 +651,11 @@ __global__ void __launch_bounds__(256)
     for (int64_t j = first; j < npix / 4; j += stride) {
       const float4 r = __ldcs(reinterpret_cast<const float4*>(x) + j);
       const float4 w = values(r);
-      if (absmax)
-        top = max(top, max(max(mag(w.x), mag(w.y)), max(mag(w.z), mag(w.w))));
       alignas(16) T v[4] = {to_store<T>(w.x), to_store<T>(w.y), to_store<T>(w.z),
                             to_store<T>(w.w)};
+      if (absmax)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) top = max(top, mag((float)v[k], nan));
       if constexpr (sizeof(T) == 4)
         reinterpret_cast<uint4*>(o)[j] = *reinterpret_cast<const uint4*>(v);
       else
@@ -687,8 +695,9 @@ __global__ void __launch_bounds__(256)
       for (int q = 0; q < 4; ++q) {
         const uint32_t at = j + 256u * (k + q);
         if (whole() || at < n) {
-          if (absmax) top = max(top, mag(v4[q]));
-          o[at + y * pad] = to_store<T>(v4[q]);
+          const T put = to_store<T>(v4[q]);
+          if (absmax) top = max(top, mag((float)put, nan));
+          o[at + y * pad] = put;
         }
         ahead(step_y, step_x);
       }
@@ -719,7 +728,7 @@ size_t sky_partial_doubles(int N) {
 
 int launch_normalize(const float* raw, int N, int W, int H, int normalize, float cr_clip,
                      int storage, void* cube, int pitch, double* mu, double* sigma,
-                     double* partial, unsigned* absmax, cudaStream_t s) {
+                     double* partial, unsigned* absmax, bool nan, cudaStream_t s) {
   const int64_t npix = (int64_t)W * H;
   int launches = 0;
   SkyPartial* parts = reinterpret_cast<SkyPartial*>(partial);
@@ -743,30 +752,30 @@ int launch_normalize(const float* raw, int N, int W, int H, int normalize, float
   switch (storage) {
     case ST_F32:
       k_normalize_store<float><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
-                                                 (float*)cube, pitch, mu, sigma, absmax);
+                                                 (float*)cube, pitch, mu, sigma, absmax, nan);
       break;
     case ST_F16:
       k_normalize_store<__half><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
-                                                  (__half*)cube, pitch, mu, sigma, absmax);
+                                                  (__half*)cube, pitch, mu, sigma, absmax, nan);
       break;
     default:
       k_normalize_store<__nv_bfloat16><<<g, 256, 0, s>>>(raw, W, H, normalize, cr_clip, state,
                                                          (__nv_bfloat16*)cube, pitch, mu, sigma,
-                                                         absmax);
+                                                         absmax, nan);
       break;
   }
   return launches + 1;
 }
 
-int launch_absmax(const float* x, int64_t n, unsigned* absmax, cudaStream_t s) {
+int launch_absmax(const float* x, int64_t n, bool nan, unsigned* absmax, cudaStream_t s) {
   const int64_t blocks = std::min((int64_t)8 * 152, (n + 4095) / 4096);
-  k_absmax<<<(unsigned)std::max((int64_t)1, blocks), 256, 0, s>>>(x, n, absmax);
+  k_absmax<<<(unsigned)std::max((int64_t)1, blocks), 256, 0, s>>>(x, n, nan, absmax);
   return 1;
 }
 
-int launch_run_margins(const FieldDev* fds, int n, const unsigned* absmax, float* margin, int* use,
-                       cudaStream_t s) {
-  k_run_margins<<<1, 256, 0, s>>>(fds, n, absmax, margin, use);
+int launch_margins(const FieldDev* fds, int n, int mode, const unsigned* absmax, float* margin,
+                   int* use, Counters* ctr, cudaStream_t s) {
+  k_margins<<<1, 256, 0, s>>>(fds, n, mode, absmax, margin, use, ctr);
   return 1;
 }
 

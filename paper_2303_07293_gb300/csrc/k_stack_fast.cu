@@ -100,6 +100,12 @@ struct FastArgs {
   float* dump_S;    // optional [nvx*nvy][H][W] of a single field (tests)
   int32_t* dump_C;
   const int* d_skip;  // non-zero: the run kernel has done the work (or NULL)
+  // bilinear sampling: how far below the threshold a sum is still kept, per
+  // field of the launch or, by field of the plan, in device memory, and 0
+  // where that is too far for this kernel (or NULL)
+  float margin[kMaxFields];
+  const float* d_margin;
+  const int* d_use;
 };
 
 __device__ int pattern_of(const int (&c)[kMB]) {
@@ -385,6 +391,7 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
   __shared__ Item item_info[kItemSlots];    // the items in flight
 
   if (p.d_skip && *p.d_skip != 0) return;  // (uniform over the grid)
+  if (BL && p.d_use && *p.d_use == 0) return;
   T* smem = reinterpret_cast<T*>(reinterpret_cast<char*>(smem_raw) +
                                  ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -951,11 +958,11 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
         for (int b = 0; b < kWords; ++b) mask[b] = 0u;
         // bilinear: the resolver re-forms each value with the generic
         // arithmetic, which differs from the factored form by FP32 rounding;
-        // the pre-filter threshold is lowered by a relative 2e-4 of the
-        // threshold's scale so no point is dropped for that reason
-        auto lower = [&](float t) {
-          return BL ? t - 2e-4f * (fabsf(t) + sqrtf((float)N)) : t;
-        };
+        // the pre-filter threshold is lowered by a bound of the difference
+        // (bilinear_margin in st_internal.h), so no point is dropped for it
+        float margin = 0.0f;
+        if constexpr (BL) margin = p.d_margin ? __ldg(p.d_margin + ff.field) : p.margin[it.f];
+        auto lower = [&](float t) { return BL ? t - margin : t; };
         if (n_full == N) {
           // interior item: every output is covered by all N frames
           const float thr_n = lower(__ldg(ff.thr + max(N, ff.nmin)));
@@ -997,6 +1004,26 @@ __device__ __forceinline__ void stack_fast_body(const FastArgs& p) {
           }
         }
         const bool col_ok = x < ff.W && av < ff.nvx;
+        if constexpr (BL) {
+          // those that reach the threshold in either arithmetic are counted:
+          // if they alone overflow the list, no other kernel's points fit
+          uint32_t any = 0u;
+#pragma unroll
+          for (int b = 0; b < kWords; ++b) any |= mask[b];
+          if (n_full == N && __any_sync(0xffffffffu, any != 0u)) {
+            const float sure = __ldg(ff.thr + max(N, ff.nmin)) + margin;
+            int count = 0;
+#pragma unroll
+            for (int j = 0; j < kMB; ++j)
+#pragma unroll
+              for (int m = 0; m < KY / 2; ++m)
+                if (it.B * kMB + j < ff.nvy)
+                  count += (int)(acc[j][m].x >= sure) + (int)(acc[j][m].y >= sure);
+            count = __reduce_add_sync(0xffffffffu, col_ok ? count : 0);
+            if (lane == 0 && count > 0)
+              atomicAdd(&p.ctr->n_sure, (unsigned long long)count);
+          }
+        }
         for (int b = 0; b < kWords; ++b) {
           uint32_t mk = col_ok ? mask[b] : 0u;
           while (__any_sync(0xffffffffu, mk != 0u)) {
@@ -1653,6 +1680,11 @@ int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, fl
   a.dump_S = dump_S;
   a.dump_C = dump_C;
   a.d_skip = runs ? rc->d_use : nullptr;
+  if (fp0->bl && rc) {
+    for (int i = 0; i < n && rc->margin; ++i) a.margin[i] = rc->margin[order[i]];
+    a.d_margin = rc->d_margin;
+    a.d_use = rc->d_use;
+  }
   const int esz = fds[0].storage == ST_F32 ? 4 : 2;
   const int stage_bytes = ((boxh * boxw * esz) + 127) & ~127;
   void (*fn)(FastArgs) = dump_S ? var.dump_fn : var.fn;

@@ -292,7 +292,8 @@ int64_t normalize_field(st_plan_t* p, int fi, const float* d_frames, bool larges
   if (!fp.d_cube) return 0;
   return launch_normalize(d_frames, fp.f.n_frames, fp.f.width, fp.f.height, p->o.normalize,
                           p->o.cr_clip, p->o.storage, fp.d_cube, fp.pitch, nullptr, nullptr,
-                          p->d_sky, largest ? p->d_absmax + fi : nullptr, p->s);
+                          p->d_sky, largest ? p->d_absmax + fi : nullptr,
+                          p->o.mode == ST_NEAREST, p->s);
 }
 
 // Tables + optional normalisation for field fi with the given frames/times.
@@ -343,14 +344,14 @@ void hold_copy(FieldPlan& fp, bool wanted) {
   }
 }
 
-// What a search's first pass took, where a second follows.
+// A search's second pass: what those before it took, and what it does else.
 struct Redo {
   double stack_ms;
   int64_t stack_launches, launches;
+  bool plain;                 // the default kernel that passes on the fewest points
+  std::vector<char> direct;   // fields that go to the direct gather
 };
 
-// redo: the second pass, with the default kernel that passes on the fewest
-// points (the pending list overflowed).
 st_status device_search(st_plan_t* p, const float* const* d_frames, const double* const* h_times,
                         st_candidate* d_out, int64_t capacity, int64_t* h_count,
                         const Redo* redo = nullptr) {
@@ -371,7 +372,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     if (changed) p->plain = false;
     fds[fi] = field_dev(p->F[fi], d_frames[fi], fi, p->o.storage);
   }
-  const bool plain = redo || p->plain;
+  const bool plain = (redo && redo->plain) || p->plain;
   // fields that fit the register-window kernel run in one persistent launch;
   // its variant is tuned (or looked up) on the field with the most work
   std::vector<char> use_fast(nf, 0);
@@ -392,7 +393,8 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
       }
     }
     // (without a copy the direct gather reads the frames as they are)
-    use_fast[fi] = fp.fast && fp.fast_fits && !(fp.copies && !fp.d_cube);
+    use_fast[fi] = fp.fast && fp.fast_fits && !(fp.copies && !fp.d_cube) &&
+                   !(redo && redo->direct[fi]);
     if (use_fast[fi]) {
       fast_fds.push_back(fds[fi]);
       fast_fps.push_back(fp.fast);
@@ -445,23 +447,31 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   }
   for (int fi = 0; fi < nf; ++fi) p->F[fi].last_variant = use_fast[fi] ? 1 : 0;
 
-  // The run kernel sums in another order than the plain definition and keeps
+  // The run kernel sums in another order than the plain definition, and the
+  // bilinear window kernel forms the samples in another way: they keep
   // points down to a margin below the threshold.  The margin follows from the
   // largest value: the clip, where there is one; else it is found on the
-  // device, which then decides between the run kernel and the one that stands
-  // in for it.  (Unnormalised FP32 frames take a pass for it: as long as 40
-  // velocities' stacks, so grids of fewer than 256 leave it.)
+  // device, which then decides between the kernel and what stands in for it.
+  // (Unnormalised FP32 frames take a pass for it: as long as 40 velocities'
+  // stacks, so grids of fewer than 256 leave the run kernel.)
+  const bool bilinear = p->o.mode == ST_BILINEAR && !fast_fds.empty();
   bool runs = !plain && !fast_fds.empty() &&
               fast_runs_chosen(fast_fds.data(), fast_fps.data(), (int)fast_fds.size());
-  const bool known = p->o.normalize && p->o.cr_clip > 0.0f;
+  const float clip = p->o.normalize ? p->o.cr_clip : 0.0f;
+  bool known = clip > 0.0f;
   std::vector<float> margin(fast_fds.size());
-  for (size_t i = 0; i < fast_fds.size() && runs; ++i) {
+  for (size_t i = 0; i < fast_fds.size() && (runs || bilinear); ++i) {
     const FieldPlan& fp = p->F[fast_fds[i].field];
     const double tau = fp.f.snr_threshold;
-    margin[i] = run_margin(1.01f * p->o.cr_clip, fp.f.n_frames,
-                           (float)(tau * std::sqrt((double)fp.f.n_frames)));
-    if (known)
-      runs = run_margin_ok(margin[i], fp.nmin, (float)(tau * std::sqrt((double)fp.nmin)));
+    // (a 16-bit value may be larger than the value it was rounded from)
+    margin[i] = margin_of(p->o.mode, 1.01f * clip, fp.f.n_frames,
+                          (float)(tau * std::sqrt((double)fp.f.n_frames)));
+    const bool small = margin_ok(p->o.mode, margin[i], fp.nmin,
+                                 (float)(tau * std::sqrt((double)fp.nmin)));
+    if (bilinear)  // (a clip beyond FP16's range does not keep infinities out)
+      known = known && small && !(p->o.storage == ST_F16 && clip > 6e4f);
+    else if (known)
+      runs = small;
     else if (!fp.d_cube)
       runs = fp.nk() >= 256;
   }
@@ -478,7 +488,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   };
   auto issue = [&](int64_t* stack_launches, int64_t* launches) -> cudaError_t {
     cudaError_t e = cudaMemsetAsync(p->d_ctr, 0, sizeof(Counters), p->s);
-    const bool largest = runs && !known;
+    const bool largest = (runs || bilinear) && !known;
     if (largest && e == cudaSuccess)
       e = cudaMemsetAsync(p->d_absmax, 0, sizeof(unsigned) * nf, p->s);
     for (int fi = 0; fi < nf; ++fi) {
@@ -488,10 +498,11 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
         *launches += normalize_field(p, fi, d_frames[fi], largest && use_fast[fi]);
       if (largest && use_fast[fi] && fds[fi].cube == d_frames[fi])
         *launches += launch_absmax(d_frames[fi], p->F[fi].P() * p->F[fi].f.n_frames,
-                                   p->d_absmax + fi, p->s);
+                                   p->o.mode == ST_NEAREST, p->d_absmax + fi, p->s);
     }
     if (largest)
-      *launches += launch_run_margins(p->d_fds, nf, p->d_absmax, p->d_margin, p->d_use, p->s);
+      *launches += launch_margins(p->d_fds, nf, p->o.mode, p->d_absmax, p->d_margin, p->d_use,
+                                  p->d_ctr, p->s);
     if (e == cudaSuccess) e = record(p->e0);
     if (!fast_fds.empty()) {
       int n = launch_stack_fast_multi(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(),
@@ -584,12 +595,36 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
   Counters c = *p->h_ctr;
   if (runs)
     fast_note_ran(fast_fds.data(), fast_fps.data(), (int)fast_fps.size(), c.runs != 0);
-  if ((c.error & ERR_PENDING_OVERFLOW) && !plain && !fast_fds.empty() &&
-      fast_plain_differs(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(), c.runs != 0)) {
-    const Redo first{p->stack_ms, p->stack_launches, L};
-    return device_search(p, d_frames, h_times, d_out, capacity, h_count, &first);
+  // ---- a second pass, where it can give another result
+  const bool over = (c.error & ERR_PENDING_OVERFLOW) != 0;
+  Redo next{p->stack_ms, p->stack_launches, L, false, std::vector<char>(nf, 0)};
+  bool again = false;
+  if (c.error & ERR_MARGIN) {
+    // fields whose margin is too wide: the direct gather
+    size_t left = 0;
+    std::vector<float> m(nf);
+    CK(cudaMemcpy(m.data(), p->d_margin, sizeof(float) * nf, cudaMemcpyDeviceToHost));
+    for (int fi = 0; fi < nf; ++fi) {
+      const FieldPlan& fp = p->F[fi];
+      next.direct[fi] = !use_fast[fi] ||
+                        !margin_ok(p->o.mode, m[fi], fp.nmin,
+                                   (float)((double)fp.f.snr_threshold *
+                                           std::sqrt((double)fp.nmin)));
+      left += next.direct[fi] == 0;
+    }
+    if (left == fast_fds.size()) next.direct.assign(nf, 1);
+    again = true;
+  } else if (over && bilinear) {
+    // the margin's points may be what does not fit
+    next.direct.assign(nf, 1);
+    again = (int64_t)c.n_sure <= p->pend_cap;
+  } else if (over && !plain && !fast_fds.empty()) {
+    next.plain = true;
+    again = fast_plain_differs(fast_fds.data(), fast_fps.data(), (int)fast_fds.size(),
+                               c.runs != 0);
   }
-  if (redo && !(c.error & ERR_PENDING_OVERFLOW)) {
+  if (again) return device_search(p, d_frames, h_times, d_out, capacity, h_count, &next);
+  if (redo && redo->plain && !over) {
     // the points fit but for the margin's: searches at these times start here
     p->plain = true;
     ++p->gen;  // (a captured graph runs the first pass)
@@ -867,7 +902,7 @@ st_status st_normalize(st_plan_t* p, int32_t field, const float* d_frames, void*
   double* d_ms = nullptr;
   CK(cudaMalloc(&d_ms, sizeof(double) * 2 * f.n_frames));
   launch_normalize(d_frames, f.n_frames, f.width, f.height, 1, p->o.cr_clip, p->o.storage, d_cube,
-                   f.width, d_ms, d_ms + f.n_frames, p->d_sky, nullptr, p->s);
+                   f.width, d_ms, d_ms + f.n_frames, p->d_sky, nullptr, false, p->s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && h_mu)
     e = cudaMemcpyAsync(h_mu, d_ms, sizeof(double) * f.n_frames, cudaMemcpyDeviceToHost, p->s);

@@ -25,9 +25,13 @@ struct Counters {
   unsigned int error;             // bit flags, ERR_*
   unsigned int runs;              // 1: the run kernel did the stacking
   unsigned long long work_next;   // persistent-kernel work counter
+  unsigned long long n_sure;      // pending points that reach the threshold for certain
+                                  // (bilinear window kernel; a lower bound)
 };
 
-enum : unsigned { ERR_PENDING_OVERFLOW = 1u, ERR_CAND_OVERFLOW = 2u, ERR_TIMEOUT = 4u };
+// ERR_MARGIN: the bilinear window kernel left the work (its margin is too wide)
+enum : unsigned { ERR_PENDING_OVERFLOW = 1u, ERR_CAND_OVERFLOW = 2u, ERR_TIMEOUT = 4u,
+                  ERR_MARGIN = 8u };
 
 // Everything a kernel needs to read one field.  Plain data, passed by value.
 struct FieldDev {
@@ -65,13 +69,14 @@ int launch_shift_tables(const double* d_t, int N, double t_ref, double vx0, doub
 // Sky statistics (FP64, deterministic) and normalisation/conversion.
 //   partial: workspace of sky_partial_doubles(N) doubles.
 size_t sky_partial_doubles(int N);
-//   cube: rows of W values, pitch values apart.
+//   cube: rows of W values, pitch values apart.  absmax, nan: as launch_absmax,
+//   of the stored values, if absmax is not NULL.
 int launch_normalize(const float* raw, int N, int W, int H, int normalize, float cr_clip,
                      int storage, void* cube, int pitch, double* mu, double* sigma,
-                     double* partial, unsigned* absmax, cudaStream_t s);
-// Largest |x| of n values that are not NaN, as FP32 bits, into *absmax (which
-// the caller zeroes; launch_normalize: of the stored values, if not NULL).
-int launch_absmax(const float* x, int64_t n, unsigned* absmax, cudaStream_t s);
+                     double* partial, unsigned* absmax, bool nan, cudaStream_t s);
+// Largest |x| of n values as FP32 bits, into *absmax (which the caller zeroes).
+// nan: a NaN counts as larger than any (else not at all).
+int launch_absmax(const float* x, int64_t n, bool nan, unsigned* absmax, cudaStream_t s);
 
 // Bound of the difference between the FP32 sum of N values of at most
 // `largest` in frame order and the run kernel's: an addition errs by at most
@@ -85,17 +90,41 @@ __host__ __device__ inline float run_margin(float largest, int N, float thr) {
   const float n = (float)N;
   return 1.02f * 0x1p-24f * (largest * n * (n + 40.0f) + 4.0f * thr);
 }
-// Whether the margin is small against the noise of the least covered points:
-// the points it adds are then at most about a tenth of those above threshold.
+// Bound of the difference between the bilinear window kernel's sum (the
+// sample as two horizontal interpolations, weighted 1 - fy and fy) and the
+// direct gather's (four taps, each weighted by a rounded product): with taps
+// of at most `largest`, the weights and interpolations of a frame err by at
+// most 2 u and 3.5 u times that, and the two and four multiply-adds by u times
+// the sum so far, i largest after i frames: u largest N (3 N + 8.5).  (The
+// last term: roundings below the normal range.)
+__host__ __device__ inline float bilinear_margin(float largest, int N, float thr) {
+  const float n = (float)N;
+  return 1.02f * 0x1p-24f * (largest * n * (3.0f * n + 9.0f) + 4.0f * thr) + n * 0x1p-146f;
+}
+// Whether the margin is at most `share` of the noise of the least covered
+// points over the threshold: it then adds about share times as many points as
+// lie above the threshold for small shares, e^share times for larger ones.
 // (False for a margin that an infinite or NaN value made.)
-__host__ __device__ inline bool run_margin_ok(float margin, int nmin, float thr_nmin) {
+__host__ __device__ inline bool margin_ok(float margin, int nmin, float thr_nmin, float share) {
   const float root = sqrtf((float)(nmin > 1 ? nmin : 1));
   const float tau = thr_nmin / root;
-  return margin * (tau > 1.0f ? tau : 1.0f) <= 0.1f * root;
+  return margin * (tau > 1.0f ? tau : 1.0f) <= share * root;
 }
-// The margins of the n fields, and whether all are small, from the largest values.
-int launch_run_margins(const FieldDev* fds, int n, const unsigned* absmax, float* margin, int* use,
-                       cudaStream_t s);
+// Shares up to which the kernels that need a margin run: the run kernel's
+// stand-in costs twice its time, the bilinear window kernel's (the direct
+// gather) ten times, and twenty times the points above a threshold of 5 are
+// still few.
+constexpr float kRunShare = 0.1f, kBilinearShare = 3.0f;
+__host__ __device__ inline float margin_of(int mode, float largest, int N, float thr) {
+  return mode == ST_BILINEAR ? bilinear_margin(largest, N, thr) : run_margin(largest, N, thr);
+}
+__host__ __device__ inline bool margin_ok(int mode, float margin, int nmin, float thr_nmin) {
+  return margin_ok(margin, nmin, thr_nmin, mode == ST_BILINEAR ? kBilinearShare : kRunShare);
+}
+// The margins of the n fields, and whether all are small enough, from the
+// largest values (bilinear sampling: else ERR_MARGIN, too).
+int launch_margins(const FieldDev* fds, int n, int mode, const unsigned* absmax, float* margin,
+                   int* use, Counters* ctr, cudaStream_t s);
 
 // Generic stack kernels over velocity indices [k0, k0+nk): threshold ->
 // pending list; optional dump of S and n_cov for the listed velocities.
@@ -137,7 +166,8 @@ bool fast_stage(const FieldDev* fds, FastPlan* const* fps, int n, bool plain, cu
 // work (k_stack_runs.cu): it keeps points
 // down to a margin below the threshold, given per field (margin, or d_margin in
 // device memory); with d_use it runs only if *d_use is not 0, else the
-// variant that stands in for it does (both are launched).
+// variant that stands in for it does (both are launched).  Bilinear sampling:
+// the window kernel keeps such a margin, and does nothing where *d_use is 0.
 struct RunCtl {
   bool runs;              // the run kernel may do the work
   const float* margin;    // host, [n] in the order of fds (NULL: 0)

@@ -84,7 +84,7 @@ def test_half_precision_values_beyond_its_range(st):
 @pytest.mark.parametrize("graph", [False, True])
 def test_one_field_of_several(st, graph):
     # the field with an infinite pixel alone goes to the direct gather
-    made = [field(96 - 3 * k, H=40 + k, seed=k, nv=9) for k in range(3)]
+    made = [field(96 - 4 * k, H=40 + k, seed=k, nv=9) for k in range(3)]
     made[1][0][5, 6, 7] = np.inf
     fr, t, f = [m[0] for m in made], [m[1] for m in made], [m[2] for m in made]
     assert lists(st, fr, t, f, use_graph=graph) == [1, 0, 1]

@@ -74,7 +74,8 @@ def test_margin_that_does_not_fit_is_found_out_once(st, graph):
 def test_overflow_is_reported_after_one_pass(st, mode, tile):
     # a few more points than the list holds: the search takes no longer than
     # one that succeeds (half as long again for the clock's sake)
-    x, t, f = field(W=512, H=512, N=48, nv=64, tau=4.7)
+    # (interpolated noise is weaker)
+    x, t, f = field(W=512, H=512, N=48, nv=64, tau=4.7 if mode == "nearest" else 3.0)
     kw = dict(mode=mode, tile=tile, normalize=True, cr_clip=10.0)
     best = {}
     for cap in (1, 1 << 22):
