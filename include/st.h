@@ -106,7 +106,8 @@ typedef struct {
                                 relative shifts once (the "runs" variant) and
                                 takes a frame-order variant for short fields;
                                 detections do not depend on the choice */
-  const char* tune_cache;    /* JSON file for autotuned tiles, or NULL */
+  const char* tune_cache;    /* JSON file for autotuned tiles, or NULL (an entry holds
+                                for the list of variants it was written for) */
   int64_t pending_capacity;  /* above-threshold points held before the local-max
                                 test; 0 selects a default of 4 Mi points */
 } st_opts;

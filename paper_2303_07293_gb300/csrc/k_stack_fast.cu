@@ -1314,6 +1314,18 @@ int fast_autotune(const FieldDev& fd, FastPlan* fp, int64_t items, Pending* pend
   cudaEventDestroy(e1);
   return launches;
 }
+uint32_t fast_list_mark(int storage, int mode) {
+  int n = 0;
+  const Variant* vars = variants_for(storage, mode == ST_BILINEAR, &n);
+  uint32_t h = 2166136261u;
+  for (int v = 0; v < n; ++v)
+    for (const char* c = vars[v].name;; ++c) {  // (with the ends of the names)
+      h = (h ^ (unsigned char)*c) * 16777619u;
+      if (!*c) break;
+    }
+  return h;
+}
+
 const char* fast_variant_name(const FastPlan* fp, int storage) {
   int n = 0;
   const Variant* vars = variants_for(storage, fp && fp->bl, &n);

@@ -207,11 +207,13 @@ st_status check_times(const double* t, int N, const st_field& f, int idx) {
 
 size_t store_bytes(int storage) { return storage == ST_F32 ? 4 : 2; }
 
-// Autotuning cache: a flat JSON object {"<field key>": variant, ...}.
+// Autotuning cache: a flat JSON object {"<field key>": variant, ...}.  A variant
+// is a place in its list, so the key ends with a mark of the list: entries
+// that were written for another one are left alone.
 std::string tune_key(const st_field& f, int storage, int mode, int sms) {
   char b[160];
-  snprintf(b, sizeof b, "W%d_H%d_N%d_nvx%d_nvy%d_st%d_m%d_sm%d", f.width, f.height, f.n_frames,
-           f.nvx, f.nvy, storage, mode, sms);
+  snprintf(b, sizeof b, "W%d_H%d_N%d_nvx%d_nvy%d_st%d_m%d_sm%d_v%08x", f.width, f.height,
+           f.n_frames, f.nvx, f.nvy, storage, mode, sms, fast_list_mark(storage, mode));
   return b;
 }
 

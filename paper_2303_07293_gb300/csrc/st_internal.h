@@ -141,6 +141,8 @@ int fast_num_variants_for(const FastPlan* fp, int storage);
 int fast_get_variant(const FastPlan* fp);
 int fast_autotune(const FieldDev& fd, FastPlan* fp, int64_t items, Pending* pend,
                   int64_t pend_cap, Counters* ctr, cudaStream_t s);
+// A hash (FNV-1a) of the names of the variants for a storage type and sampling.
+uint32_t fast_list_mark(int storage, int mode);
 const char* fast_variant_name(const FastPlan* fp, int storage);
 void fast_set_variant(FastPlan* fp, int v);
 // Whether the field can use the fast kernel at all (row pitch a multiple of
