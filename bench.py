@@ -51,7 +51,7 @@ METRIC = "G pixel*frame*velocity adds/s (2048x2048x256, 801x801 grid)"
 # removed, so only a change of the code itself retires the figure): reported
 # only while the code is that one.
 STACK_TRAFFIC = {
-    ("speculoos", "f32", "nearest", "float_runs_ky8_x4_s3_f16"):
+    ("speculoos", "f32", "nearest", "float_runs_ky8_x4_s2_f16"):
         (263.554441728e9 + 26.86097664e9, "236fdd105713"),
 }
 

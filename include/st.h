@@ -103,9 +103,13 @@ typedef struct {
                                 field whose motion does not fit the window takes
                                 the direct-gather kernel.  The default for
                                 nearest sampling adds frames with equal
-                                relative shifts once (the "runs" variant) and
-                                takes a frame-order variant for short fields;
-                                detections do not depend on the choice */
+                                relative shifts once (the "runs" variant, twice
+                                as fast) and takes a frame-order variant, for
+                                all fields of the plan, where they are short or
+                                small, where one field's motion does not fit its
+                                windows, or where values are too large (or not
+                                finite) for its rounding margin; detections do
+                                not depend on the choice */
   const char* tune_cache;    /* JSON file for autotuned tiles, or NULL (an entry holds
                                 for the list of variants it was written for) */
   int64_t pending_capacity;  /* above-threshold points held before the local-max

@@ -272,7 +272,6 @@ def render():
             out.append(f'  "{ln}\\n\\t" \\')
         out.append("")
     ops = ", ".join(f'"+l"(s[{k}])' for k in range(VEL * PAIRS))
-    ops = ", ".join(f'"+l"(s[{k}])' for k in range(VEL * PAIRS))
     out.append("#define ST_RUN_OPERANDS(s, slot, ph, off, stages, base, words, lane, tm) \\")
     out.append(f'  : {ops}, "+r"(slot), "+r"(ph), "+r"(off) \\')
     out.append('  : "r"(stages), "r"(base), "r"(words), "r"(lane), "r"(tm) : "memory"')

@@ -1083,10 +1083,11 @@ struct Variant {
   int halves;  // x-velocity tiles per item (boxes per frame)
   int xpw;     // x-velocities per thread (2: a half holds two table tiles)
   const char* name;
-  bool runs = false;  // the run kernel (k_stack_runs.cu)
+  bool runs = false;  // the run kernel (k_stack_runs.cu: 8 rows, 4 x-velocities a
+                      // group, a ring of 2 stages of 16 frames)
 };
 #define RUNS(T) \
-  {nullptr, nullptr, 0, 0, 16, 0, kTX, 4, 1, #T "_runs_ky8_x4_s3_f16", true}
+  {nullptr, nullptr, 0, 0, 16, 0, kTX, 4, 1, #T "_runs_ky8_x4_s2_f16", true}
 
 #define ST_VARIANT(T, KY, S, F, BL, CP, OPT, H)                                               \
   {                                                                                           \
@@ -1651,7 +1652,8 @@ int launch_stack_fast_multi(const FieldDev* fds, FastPlan* const* fps, int n, fl
       total += run_items(fps[order[i]]->h_ff);
     }
     r.n_fields = n;
-    // (autotuning: 32 x 16 pixels and about 32 x-velocities an item)
+    // (autotuning: an item has 32 x 32 pixels and up to 16 x-velocities, four
+    // times the 32 x 16 and 8 that the limit counts)
     const int64_t limit = (fp0->item_limit + 3) / 4;
     r.n_items = limit > 0 && total > limit ? limit : total;
     r.d_margin = rc->d_margin;

@@ -33,7 +33,7 @@ struct FastField {
   const int* cov_ymax;
   int cov_len;
   // tables of the run kernel (k_stack_runs.cu)
-  int nG, nT;           // groups of 4 x-velocities, tiles of at most 8 groups
+  int nG, nT;           // groups of 4 x-velocities, tiles of at most 4 groups
   const uint32_t* xg;   // [N][nG] shift and steps of a group
   const int2* ord;      // [nB][N] frames by pattern
 };

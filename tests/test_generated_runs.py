@@ -113,3 +113,28 @@ def test_steps_move_the_sum_from_one_offset_to_the_next():
             pair = k // 2 * 2
             assert acc[k] == (("acc", pair), ("acc", pair + 1), ("add", plus), ("sub", minus))
             assert first[k] == (plus, ("sub", minus))
+
+
+def test_pattern_words_give_each_patterns_offsets():
+    # the instructions between a frame that ends a run and the step loop, run
+    # on that frame's word for every pattern of the next run
+    g = _gen()
+    for dtype in g.DTYPES:
+        lines = g.item_loop(dtype)
+        k = lines.index("@pl bra.uni RKEEP;", lines.index("RNEXT:")) + 1
+        code = lines[k:lines.index("RSTEP:")]
+        for pid in range(15):
+            reg = {"sn": pid << g.PAT_BIT | 1 << g.END_BIT | 0x155, "pl": None}
+
+            def val(t):
+                return reg[t] if t in reg else int(t, 0) & 0xffffffff
+            for ln in code:
+                op, rest = ln.rstrip(";").split(" ", 1)
+                d, *a = [t.strip() for t in rest.split(",")]
+                v = [bool(reg[t]) if t == "pl" else val(t) for t in a]
+                reg[d] = {"shr.u32": lambda: v[0] >> v[1], "and.b32": lambda: v[0] & v[1],
+                          "setp.lt.u32": lambda: v[0] < v[1], "setp.eq.u32": lambda: v[0] == v[1],
+                          "selp.b32": lambda: v[0] if v[2] else v[1]}[op]()
+            assert [reg["st0"] >> (2 * j) & 3 for j in range(4)] == \
+                [g.pat_off(pid, j) for j in range(4)], pid
+            assert reg["st0"] < 256
