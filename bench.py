@@ -54,6 +54,24 @@ STACK_TRAFFIC = {
     ("speculoos", "f32", "nearest", "float_runs_ky8_x4_s2_f16"):
         (263.554441728e9 + 26.86097664e9, "236fdd105713"),
 }
+# Shared-memory wavefronts (one a clock and SM) per addition of the plain
+# definition, the run kernel's own bound: one ncu capture of
+# `l1tex__data_pipe_lsu_wavefronts_mem_shared.sum` on the same field with
+# 101 x 101 velocities (same file), with the code's hash.
+STACK_WAVEFRONTS = {
+    ("speculoos", "f32", "nearest", "float_runs_ky8_x4_s2_f16"):
+        (44822230033 / (2048 * 2048 * 256 * 101 * 101), "236fdd105713"),
+}
+
+
+def own_bound(key, adds_per_s, sms, mhz):
+    """The fraction of the run kernel's own bound that a rate of plain
+    additions comes to (None: not captured on this code)."""
+    w = STACK_WAVEFRONTS.get(key)
+    if not w or w[1] != stack_source_sha(key[3]):
+        return None
+    return {"bound": "shared-memory wavefronts", "frac": adds_per_s * w[0] / (sms * mhz * 1e6),
+            "wavefronts_per_4096_adds": 4096 * w[0]}
 
 
 def stack_source_sha(variant="_runs_"):
@@ -768,7 +786,10 @@ def main():
             "work_per_unit": per_unit,
             "work_note": "adds of the plain definition, N per pixel and velocity; the runs "
                          "variant sums frames with equal relative shifts once and makes "
-                         "fewer than a third of them, so frac can exceed 1",
+                         "fewer than a third of them, so frac can exceed 1: its own bound is "
+                         "own_bound",
+            "own_bound": own_bound((args.workload, args.storage, args.mode, variant),
+                                   achieved * 1e12 / per_unit, sms, max_mhz),
             "kernel": "stack (shift-and-stack + threshold)", "launches_per_step":
                 stack_launch / args.steps, "avg_launch_ms": stack_avg_ms,
             "peak_basis": f"{sms} SMs x 128 FP32 lanes x {max_mhz:.0f} MHz (max SM clock)"}

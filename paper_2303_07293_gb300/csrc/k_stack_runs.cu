@@ -43,8 +43,8 @@
 // wavefront each), 18 paired adds and 15 other instructions, against 64
 // paired adds at the FP32 pipe's rate alone; 86 instructions in all on 64
 // frames, 75 on 256 (the ends of runs, stages and items are the rest), issue
-// slots 56 % and shared-memory wavefronts 43 to 46 % busy on 64 frames, where warps
-// wait for the slowest at each stage.  Measured against the frame-order kernel
+// slots 53 % and shared-memory wavefronts 43 % busy on 64 frames (58 % on 256), where
+// warps wait for the slowest at each stage.  Measured against the frame-order kernel
 // (rates in additions of the plain definition, 40.3 T/s the FP32 pipe's):
 // 1024^2 x 64, 161^2 velocities 86.7 -> 56.7 ms (30.7 T/s); 2048^2 x 256, 101^2
 // 491 -> 246 ms (44.6 T/s); six FP16 fields of 46..120 frames, 61^2 85.7 -> 47.5
