@@ -28,8 +28,8 @@
 // Membership is a comparison with the first and last FP32 value that the
 // FP64 rule keeps.  A sample of the frame gives p and r of the first pass,
 // the statistics of each pass those of the next.
-// Measured on a 2048^2 x 256 FP32 cube (4.29 GB): a pass 1.18 ms, 3.6 TB/s
-// (issue slots: 34 instructions a pixel), the statistics 5.9 ms; with FP64
+// Measured on a 2048^2 x 256 FP32 cube (4.29 GB): a pass 1.15 ms, 3.7 TB/s
+// (issue slots: 33 instructions a pixel), the statistics 5.8 ms; with FP64
 // sums they took 104 ms in 6 passes.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -222,16 +222,16 @@ struct Codes {
     float2 t = __fadd2_rn(ds, m1);
     d1 += bits(t);
     d2 += bits(__fadd2_rn(__fadd2_rn(ds, __ffma2_rn(t, neg, m1)), m2));
-    const float2 s = __fmul2_rn(ds, ds);
-    float2 e = __ffma2_rn(ds, ds, make_float2(-s.x, -s.y));
+    // (an fma, so that the rounded square and a sum after it stay two operations)
+    const float2 s = __ffma2_rn(ds, ds, make_float2(0.0f, 0.0f));
     t = __fadd2_rn(s, m1);
     s1 += bits(t);
-    const float2 rest = __fadd2_rn(s, __ffma2_rn(t, neg, m1));
-    t = __fadd2_rn(rest, m2);
+    const float2 a = __ffma2_rn(t, neg, m1);  // -(s on the first grid)
+    t = __fadd2_rn(__fadd2_rn(s, a), m2);
     s2 += bits(t);
-    // (what a square below 2^-22 has beyond the second grid: ties between
-    // grid points would all round one way)
-    e = __fadd2_rn(e, __fadd2_rn(rest, __ffma2_rn(t, neg, m2)));
+    // the square less both parts: its rounding error and what a square below
+    // 2^-22 has beyond the second grid (ties there would all round one way)
+    const float2 e = __ffma2_rn(ds, ds, __fadd2_rn(a, __ffma2_rn(t, neg, m2)));
     t = __fadd2_rn(e, m3);
     s3 += bits(t);
     s4 += bits(__fadd2_rn(__fadd2_rn(e, __ffma2_rn(t, neg, m3)), m4));
@@ -365,40 +365,43 @@ __device__ __forceinline__ SkyPartial sky_sums(const SkyFrame& f, int v0, int v1
   return a;
 }
 
-// Sums of two FP64 numbers that stay apart: hi + lo, lo the rounding of hi.
-struct Wide {
-  double hi, lo;
-};
-__device__ __forceinline__ Wide wide_add(Wide a, double b) {
-  const double s = __dadd_rn(a.hi, b), z = __dsub_rn(s, a.hi);
-  const double e = __dadd_rn(__dsub_rn(a.hi, __dsub_rn(s, z)), __dsub_rn(b, z));
-  return {s, __dadd_rn(a.lo, e)};
+// v 2^e, v >= 0, rounded once.
+__device__ __forceinline__ double scaled(__int128 v, int e) {
+  if (v <= 0) return 0.0;
+  const unsigned long long hi = (unsigned long long)(v >> 64), lo = (unsigned long long)v;
+  if (hi == 0) return ldexp((double)lo, e);
+  const int up = __clzll((long long)hi);
+  // the first 64 bits, the last of them set if any beyond is
+  const unsigned long long top = up ? hi << up | lo >> (64 - up) : hi;
+  return ldexp((double)(top | (unsigned long long)((lo << up) != 0)), e + 64 - up);
 }
 
-// Mean and deviation of a kept set from its sums.  The variance is a
-// difference of two terms that are up to 10^2 times as large (a pivot of 0
-// beside a mean of up to 10 deviations), so they are formed to twice FP64's
-// length: its root is the correctly rounded one but for a last place, as a
-// sum about the mean gives it.
+// Mean and deviation of a kept set from its sums.  About a pivot of 0 beside a
+// mean of up to 10 deviations the variance is a difference of terms 10^2
+// times as large, so the sums are first moved, as the integers that they
+// are, to within a step of 2^-22 of the mean: the variance is rounded twice and
+// its root once, as good as a sum about the mean.  (FP64 here is one thread's,
+// at the end of every pass: sums of twice FP64's length took 6 us a pass more.)
 __device__ void sky_moments(const SkyPartial& a, SkyState& st) {
   const double cnt = (double)a.n;
-  Wide d{ldexp((double)a.d1, st.r - 22), 0.0};
-  d = wide_add(d, ldexp((double)a.d2, st.r - 45));
-  d = wide_add(d, a.w1);
-  Wide s{ldexp((double)a.s1, 2 * st.r - 22), 0.0};
-  s = wide_add(s, ldexp((double)a.s2, 2 * st.r - 45));
-  s = wide_add(s, ldexp((double)a.s3, 2 * st.r - 47));
-  s = wide_add(s, ldexp((double)a.s4, 2 * st.r - 70));
-  s = wide_add(s, a.w2);
-  // mean = (m + ml) about the pivot; n times the variance = s - d (m + ml)
-  const double m = __ddiv_rn(__dadd_rn(d.hi, d.lo), cnt);
-  const double ml =
-      __ddiv_rn(__dadd_rn(__fma_rn(-m, cnt, d.hi), d.lo), cnt);
-  const double q = __dmul_rn(d.hi, m);
-  const double ql = __fma_rn(d.hi, m, -q) + (__dmul_rn(d.hi, ml) + __dmul_rn(d.lo, m));
-  const Wide v = wide_add(s, -q);
-  const double var = (v.hi + (v.lo - ql)) / cnt;
-  st.mu = st.pivot + (m + ml);
+  const long long c = (long long)rintf((float)a.d1 / (float)a.n);         // 2^-22
+  const __int128 d = (__int128)a.d1 * (1 << 23) + a.d2;                   // 2^-45
+  const __int128 s = ((__int128)a.s1 * (1 << 23) + a.s2) * (1 << 25) +
+                     (__int128)a.s3 * (1 << 23) + a.s4;                   // 2^-70
+  const double dc = (double)(long long)(d - (__int128)a.n * c * (1 << 23));
+  __int128 sc = s - d * c * 16 + (__int128)a.n * (c * c) * (1 << 26);
+  double m1 = dc / cnt, var;                                              // 2^-45
+  if (a.w2 == 0.0) {
+    sc -= __double2ll_rn(m1 * dc * 0x1p-20);
+    var = scaled(sc, 2 * st.r - 70) / cnt;
+    m1 = ldexp(fma(m1, 0x1p-23, (double)c), st.r - 22);
+  } else {
+    const double at = ldexp((double)c, st.r - 22);
+    m1 = (ldexp(dc, st.r - 45) + a.w1) / cnt;
+    var = (scaled(sc, 2 * st.r - 70) + (a.w2 - 2.0 * at * a.w1)) / cnt - m1 * m1;
+    m1 += at;
+  }
+  st.mu = st.pivot + m1;
   st.sigma = sqrt(var > 0.0 ? var : 0.0);
 }
 
