@@ -413,7 +413,7 @@ st_status device_search(st_plan_t* p, const float* const* d_frames, const double
     CK(cudaMemcpyAsync(p->d_fds, fds.data(), sizeof(FieldDev) * nf, cudaMemcpyHostToDevice, p->s));
     p->h_fds = fds;
   }
-  if (tune_fi >= 0 && p->o.tile == -1) {
+  if (tune_fi >= 0 && p->o.tile == -1 && !redo) {  // (a second pass keeps the variant)
     FieldPlan& tp = p->F[tune_fi];
     if (!tp.tuned) {
       const std::string key = tune_key(tp.f, fds[tune_fi].storage, p->o.mode, p->sms);

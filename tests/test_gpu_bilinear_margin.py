@@ -116,3 +116,21 @@ def test_list_that_holds_the_points_but_not_the_margin(st):
     with st.Plan(f, mode="bilinear", pending_capacity=lo) as p:
         for _ in range(2):
             assert p.candidates(x, t).tobytes() == want.tobytes()
+
+
+def test_autotuned_plan_keeps_its_variant_in_a_second_pass(st, tmp_path):
+    # the field that the variant was tuned on goes to the direct gather; the
+    # other one is not tuned for it
+    import json
+    made = [field(96, H=60 - 20 * k, N=32, seed=k, nv=12) for k in range(2)]
+    made[0][0][5, 6, 7] = np.inf
+    x, t, f = ([torch.from_numpy(m[0]).cuda() for m in made], [m[1] for m in made],
+               [m[2] for m in made])
+    cache = tmp_path / "tune.json"
+    with st.Plan(f, mode="bilinear", tile=1) as p:
+        want = p.candidates(x, t)
+    with st.Plan(f, mode="bilinear", tile=-1, tune_cache=str(cache)) as p:
+        for _ in range(2):
+            assert p.candidates(x, t).tobytes() == want.tobytes()
+            assert [p.last_stack_variant(k) for k in range(2)] == [0, 1]
+    assert len(json.loads(cache.read_text())) == 1
